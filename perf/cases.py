@@ -176,7 +176,7 @@ def _scan(r: _Rand, n):
         size, ratios = h.uniform(0.1, 1.0), [h.uniform(0.5, 1.0) for _ in range(3)]
         ax = [0.5 * size * q / max(ratios) for q in ratios]
         e1, e2 = h.uniform(0.3, 1.5), h.uniform(0.3, 1.5)
-        rot, _q = torch.linalg.qr(r.normal(3, 3))
+        rot = torch.linalg.qr(r.normal(3, 3).cpu())[0].to(r.dev)
         centre = r.uniform(3, lo=-1.0, hi=1.0)
         p = points(grid_e, grid_o, ax, e1, e2)
         area = torch.linalg.cross(p[1:, :-1] - p[:-1, :-1], p[:-1, 1:] - p[:-1, :-1]).norm(dim=-1)
