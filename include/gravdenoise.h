@@ -161,7 +161,8 @@ int denoise_set_profiling(denoise_ctx *ctx, int enable);   /* per-stage CUDA eve
  *                    A smaller value shrinks each CTA's shared memory so that
  *                    more CTAs fit per SM.  Rounded down to a power of two,
  *                    at least 64; 0 (default) = the leaf capacity.
- *  leaf_threads      threads of a per-leaf CTA: 64 or 128 (0 = default 128).
+ *  leaf_threads      threads of a per-leaf CTA: 64 or 128 (0 = default: chosen
+ *                    by the number of points and the leaf size, 64 to 512).
  *                    64 suits workloads of many small leaves (fewer idle
  *                    warps per leaf); other values give E_INVAL.
  * The autotuner (paper_2512_10386_gb300/autotune.py) picks both together with

@@ -286,6 +286,7 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   la.threads = c->leaf_threads;
   la.spin_limit = c->wait_limit;
   const int kmax = leaf_kmax(p.k);
+  la.kmax = kmax;
   la.lmax = leaf_pick_lmax(p.leaf_capacity, kmax, c->smem_optin - 2048);
   if (c->leaf_smem_points) {
     uint32_t l = 64;

@@ -201,7 +201,8 @@ struct LeafArgs {
   TrainCache train;
   int use_train;
   uint32_t ctas_per_sm;         // 0 = occupancy limit
-  uint32_t threads;             // threads per leaf CTA: 64 or 128 (0 = 128)
+  uint32_t threads;             // threads per leaf CTA: 64, 128, 256 or 512 (0 = 128)
+  int kmax;                     // leaf_kmax(p.k): rows of a spilled leaf's neighbour table
   uint32_t spin_limit;          // iterations of the bounded bulk-copy wait (0 = kSpinLimit)
   uint32_t part;                // leaves taken from the order: 0 all, 1 those before split_leaf, 2 the rest
   // cross-leaf kNN (denoise_params.cross_leaf): phase 1 runs the voxel gate only and
@@ -235,7 +236,7 @@ struct XleafArgs {
 int launch_xleaf_knn(const XleafArgs &a, int num_sms, cudaStream_t st, int *launches);
 
 int leaf_kmax(uint32_t k);
-size_t leaf_smem_bytes(uint32_t lmax, int kmax);
+size_t leaf_smem_bytes(uint32_t lmax, int kmax, int threads);
 uint32_t leaf_big_bpp(int kmax);
 uint32_t leaf_pick_lmax(uint32_t leaf_capacity, int kmax, size_t smem_limit);
 // Eq. 10-11 per leaf (box origin lo and voxel size h into the leaf table) and the

@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(256) k_leaf_order(const Leaf *__restrict__ lea
 // ---------------------------------------------------------------------------
 int leaf_kmax(uint32_t k) { return k <= 8 ? 8 : k <= 16 ? 16 : k <= 32 ? 32 : 64; }
 
-size_t leaf_smem_bytes(uint32_t lmax, int kmax) {
-  return carve<uint16_t>(nullptr, lmax, kmax, nullptr);
+size_t leaf_smem_bytes(uint32_t lmax, int kmax, int threads) {
+  return carve<uint16_t>(nullptr, lmax, kmax, threads, nullptr);
 }
 
 namespace {
@@ -161,7 +161,7 @@ namespace {
 uint32_t big_bpp_scan(int kmax) {
   size_t worst = 4u * ((kLeafSmemMax + 31u) / 32u);
   for (uint32_t cap = 65; cap <= 65536; ++cap) {
-    const size_t b = carve<uint32_t>(nullptr, cap, kmax, nullptr);
+    const size_t b = carve<uint32_t>(nullptr, cap, kmax, 128, nullptr);
     const size_t per = (b + cap - 1) / cap;
     if (per > worst) worst = per;
   }
@@ -180,7 +180,7 @@ uint32_t leaf_big_bpp(int kmax) {
 uint32_t leaf_pick_lmax(uint32_t leaf_capacity, int kmax, size_t smem_limit) {
   const uint32_t cap = leaf_capacity < 64 ? 64 : (leaf_capacity > kLeafSmemMax ? kLeafSmemMax : leaf_capacity);
   uint32_t l = pow2ceil(cap);
-  while (l > 64 && leaf_smem_bytes(l, kmax) > smem_limit) l >>= 1;
+  while (l > 64 && leaf_smem_bytes(l, kmax, 512) > smem_limit) l >>= 1;
   return l;
 }
 
@@ -192,21 +192,46 @@ int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launc
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_leaf(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches, cudaStream_t side, cudaEvent_t fork,
+// Threads of a leaf CTA where the caller leaves the choice open.  A leaf is one
+// CTA's work, so a call takes at least the time of its largest leaf; a wider CTA
+// shortens that (32 queries a warp) but waits longer at the leaf's barriers and
+// leaves fewer CTAs per SM to fill the waits.  Wide CTAs therefore pay while the
+// points are too few to keep every SM busy, or where one leaf's shared memory
+// leaves room for one to three CTAs per SM anyway.  Measured, us a call (K = 24,
+// dense scans unless noted; leaf CTAs of 128 / 256 / 512 threads):
+//   up to 64-point leaves: 64 threads, 300k points 376 -> 289
+//   256-point leaves:  40k 148 / 136 / 165, 70k (LiDAR) 159 / 155 / 223, 100k 158 / 177 / 289
+//   512-point leaves:  40k 229 / 185 / 162, 100k 270 / 232 / 228, 130k (LiDAR) 299 / 242 / 272,
+//                      200k 291 / 231 / 368, 300k 294 / 292 / 463, 560k 402 / 484 / 886
+//   1,024-point leaves: 200k 672 / 527 / 377, 300k 671 / 508 / 457, 560k 753 / 589 / 747
+//   2,048-point leaves: 10k 1184 / 838 / 661, 560k 2362 / 1612 / 1299
+static uint32_t leaf_auto_threads(uint32_t n, uint32_t lmax) {
+  if (lmax <= 64) return 64;
+  if (lmax <= 128) return 128;
+  if (lmax <= 256) return n <= (64u << 10) ? 256 : 128;
+  if (lmax <= 512) return n <= (96u << 10) ? 512 : n <= (280u << 10) ? 256 : 128;
+  if (lmax <= 1024) return n <= (384u << 10) ? 512 : 256;
+  return 512;
+}
+
+int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launches, cudaStream_t side, cudaEvent_t fork,
                 cudaEvent_t join) {
+  LeafArgs a = args;
+  if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a.n, a.lmax);
   if (a.xphase != 0) {  // the cross-leaf phases: their own instantiation
     if (launches) ++*launches;
     return launch_leaf_xl(a, num_sms, st);
   }
   auto go = [&](const LeafArgs &x, cudaStream_t s) {
-    return (x.use_dbg || x.use_train) ? launch_leaf_rec(x, num_sms, s) : launch_kmax<false, false>(x, num_sms, s);
+    return (x.use_dbg || x.use_train) ? launch_leaf_rec(x, num_sms, s) : launch_threads<false, false>(x, num_sms, s);
   };
   // A small leaf's per-leaf steps keep few warps busy; on 64-thread CTAs of a
   // 64-point shared-memory layout twice as many CTAs share an SM.  The large
   // leaves keep their 128-thread CTAs; the two launches run side by side, and the
   // small-leaf CTAs take the SMs the large-leaf CTAs leave (the order of the
   // leaves and every result are the same as with one launch).
-  const bool split = side && fork && join && a.threads != 64 && a.lmax > kSmallLeaf && a.ctas_per_sm == 0;
+  const bool split = side && fork && join && (a.threads == 0 || a.threads == 128) && a.lmax > kSmallLeaf &&
+                     a.ctas_per_sm == 0;
   if (!split) {
     if (launches) ++*launches;
     return go(a, st);

@@ -12,8 +12,7 @@
 
 namespace gd {
 
-constexpr int kLeafThreads = 128;
-constexpr int kLeafWarps = kLeafThreads / 32;
+constexpr int kLeafMaxWarps = 16;  // of the widest leaf CTA (512 threads)
 constexpr unsigned long long kEmpty = ~0ull;
 constexpr unsigned long long kInvalid = ~0ull - 1ull;
 // P_1 is followed by kPad NaN points: the kNN passes read whole steps of 4, 16
@@ -42,14 +41,14 @@ struct LeafMem {
   unsigned long long *hkey;  // [hcap] voxel hash keys
   uint32_t *hcnt;            // [hcap] voxel occupancy
   unsigned long long *sbuf;  // [scap] sort buffer
-  uint32_t *pend;            // [kSelBuf][kLeafThreads] parked boundary-bucket keys (shared memory, both paths)
+  uint32_t *pend;            // [kSelBuf][threads of the CTA] parked boundary-bucket keys (shared memory, both paths)
   float *r2, *wa;            // [cap] per P_1 position: r_K^2, (alpha/2) ell; wa also holds voxel hash slots
   float *F;                  // [cap] score; shares r2's storage (F_i is written after r2_i's last read)
   uint8_t *flag;             // [cap] 0 removed by density gate, 1 scored, 2 kept
   uint32_t *spos;            // [cap] leaf offset of each P_1 point (cross-leaf mode)
   uint32_t *cmask;           // [cap] the chunks of a query's bitmap row that hold neighbours (shares spos:
                              // the cross-leaf mode, which reads spos later, runs no kNN in this kernel)
-  void *nbr;                 // neighbours: bitmaps (shared-memory path, see bitmap_words) or [KMAX][cap] u32 (global)
+  void *nbr;                 // neighbours: bitmaps (shared-memory path, see bitmap_words) or [kmax][cap] u32 (global)
   uint32_t nbr_bytes;        // bytes of the region that holds nbr
   uint32_t hcap, scap, cap;
 };
@@ -73,8 +72,9 @@ __host__ __device__ __forceinline__ uint32_t bitmap_words(uint32_t n1) { return 
 // (the lifetimes do not overlap) the neighbour table.  Region R holds a
 // shared-memory leaf's raw points (voxel gate), then the parked kNN keys, then
 // the sort buffer of the order statistics.
+// (`threads`: threads of the CTA, which set the size of the parking area.)
 template <typename IdxT>
-__host__ __device__ __forceinline__ size_t carve(unsigned char *base, uint32_t cap, int kmax, LeafMem *m) {
+__host__ __device__ __forceinline__ size_t carve(unsigned char *base, uint32_t cap, int kmax, int threads, LeafMem *m) {
   constexpr bool kSmem = sizeof(IdxT) == 2;
   const uint32_t hcap = pow2ceil(2 * cap), scap = pow2ceil(cap);
   const size_t hash_end = al16((size_t)hcap * 8) + al16((size_t)hcap * 4);
@@ -82,7 +82,7 @@ __host__ __device__ __forceinline__ size_t carve(unsigned char *base, uint32_t c
   size_t o = al16(hash_end > nbr_bytes ? hash_end : nbr_bytes);
   size_t rbytes = (size_t)scap * 8;
   if (kSmem) {
-    const size_t raw = (size_t)cap * 16, park = (size_t)kSelBuf * kLeafThreads * 4;
+    const size_t raw = (size_t)cap * 16, park = (size_t)kSelBuf * threads * 4;
     if (raw > rbytes) rbytes = raw;
     if (park > rbytes) rbytes = park;
   }
@@ -128,8 +128,7 @@ struct LeafShared {
   float lo[3], h, delta, r2ref, Lref;
   float lshift;  // cross-leaf mode: ell_j = log2(rho_j) - lshift for a neighbour j of any leaf
   double rho_med;
-  uint32_t wsum[kLeafWarps];
-  uint32_t red[kLeafWarps][6];
+  uint32_t wsum[kLeafMaxWarps];
 };
 
 // ---------------------------------------------------------------------------
@@ -491,7 +490,7 @@ __device__ __forceinline__ void write_point(const LeafArgs &A, uint32_t g, uint8
 // ---------------------------------------------------------------------------
 // one leaf
 // ---------------------------------------------------------------------------
-template <int KMAX, typename IdxT, bool kRec, bool kXl>
+template <int kNT, typename IdxT, bool kRec, bool kXl>
 __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__restrict__ pts, const LeafMem &M,
                              LeafShared &S) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -843,7 +842,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
           const uint32_t ju = c0 + (uint32_t)(__ffs(pm) - 1);
           pm &= pm - 1u;
           const int32_t db = __float_as_int(sqdist(xq, yq, zq, X[ju], Y[ju], Z[ju]));
-          pend[(slot++) * kLeafThreads + tid] = ((uint32_t)(db - kbase) << pbits) | ju;
+          pend[(slot++) * kNT + tid] = ((uint32_t)(db - kbase) << pbits) | ju;
         }
       }
       if (act && (a != cut.c_below || np != cut.c_at)) atomicOr(&A.ctr->status, kStInternal);  // passes agree
@@ -855,7 +854,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         uint32_t K[kSelBuf];
 #pragma unroll
         for (int i = 0; i < (int)kSelBuf; ++i)
-          K[i] = (parked && (uint32_t)i < np) ? pend[i * kLeafThreads + tid] : 0xFFFFFFFFu;
+          K[i] = (parked && (uint32_t)i < np) ? pend[i * kNT + tid] : 0xFFFFFFFFu;
         // with at most 8 parked keys in every lane of the warp (the usual case) the
         // padding keys above them stay in place: a network on the first 8 suffices
         if (__reduce_max_sync(0xFFFFFFFFu, parked ? np : 0u) <= kSelBuf / 2) regsort_head<kSelBuf / 2>(K);
@@ -864,7 +863,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
 #pragma unroll
         for (int i = 0; i < (int)kSelBuf; ++i) {
           th_off = ((uint32_t)i + 1u == need) ? (K[i] >> pbits) : th_off;
-          if (parked) pend[i * kLeafThreads + tid] = K[i];  // sorted, for the emission loop below
+          if (parked) pend[i * kNT + tid] = K[i];  // sorted, for the emission loop below
         }
         uint32_t n_lt = 0, n_eq = 0;
 #pragma unroll
@@ -880,17 +879,17 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
           take = (n_lt >= 32u) ? 0xFFFFFFFFu : ((1u << n_lt) - 1u);
 #pragma unroll 1
           for (uint32_t i = n_lt; i < n_lt + n_eq; ++i) {
-            const uint32_t gi = W[pend[i * kLeafThreads + tid] & pmask];
+            const uint32_t gi = W[pend[i * kNT + tid] & pmask];
             uint32_t before = 0;
 #pragma unroll 1
-            for (uint32_t j = n_lt; j < n_lt + n_eq; ++j) before += W[pend[j * kLeafThreads + tid] & pmask] < gi;
+            for (uint32_t j = n_lt; j < n_lt + n_eq; ++j) before += W[pend[j * kNT + tid] & pmask] < gi;
             if (before < need_eq) take |= 1u << i;
           }
         }
         while (take) {
           const uint32_t i = (uint32_t)(__ffs(take) - 1);
           take &= take - 1u;
-          const uint32_t key = pend[i * kLeafThreads + tid], ju = key & pmask;
+          const uint32_t key = pend[i * kNT + tid], ju = key & pmask;
           if constexpr (kPacked) set_bit(ju);
           emit(a++, ju, W[ju], __int_as_float(kbase + (int32_t)(key >> pbits)));
         }
@@ -1276,22 +1275,23 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, uint32_t
   return false;
 }
 
-// Persistent CTAs of 128 threads, GD_LEAF_MIN_CTAS per SM for K <= 32 (a
-// 512-point leaf takes 33 KB of shared memory, so 6 fit; the register bound
-// follows from the count).  kRec: the debug / training outputs are written (a
-// separate instantiation, so that the plain path carries none of their code).
-#ifndef GD_LEAF_MIN_CTAS
-#define GD_LEAF_MIN_CTAS 6
-#endif
-template <int KMAX, bool kRec, bool kXl>
-__global__ void __launch_bounds__(kLeafThreads, (KMAX >= 64) ? 1 : GD_LEAF_MIN_CTAS) k_leaf(const LeafArgs A) {
+// Persistent CTAs of kNT threads (128, 256 or 512, see leaf_auto_threads; a 64-thread
+// launch uses the 128-thread code).  128 threads: 6 CTAs per SM, which a 512-point
+// leaf's 35 KB of shared memory allow, at 80 registers a thread; the wider CTAs
+// keep about as many warps per SM, or serve a grid that is too small to fill the
+// GPU and whose time is that of its largest leaf.  kRec: the debug / training
+// outputs are written (a separate instantiation, so that the plain path carries
+// none of their code).
+constexpr int leaf_min_ctas(int threads) { return threads <= 128 ? 6 : threads <= 256 ? 3 : 1; }
+template <int kNT, bool kRec, bool kXl>
+__global__ void __launch_bounds__(kNT, leaf_min_ctas(kNT)) k_leaf(const LeafArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) unsigned long long s_mbar;
   __shared__ LeafShared S;
   const uint32_t tid = threadIdx.x;
   const uint32_t lmax = A.lmax;
   LeafMem Ms;
-  carve<uint16_t>(smem, lmax, KMAX, &Ms);
+  carve<uint16_t>(smem, lmax, A.kmax, kNT, &Ms);
   float4 *const s_pts = Ms.raw;  // the raw points land here, P_1 is compacted out of them
   const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
   if (tid == 0) {
@@ -1332,45 +1332,44 @@ __global__ void __launch_bounds__(kLeafThreads, (KMAX >= 64) ? 1 : GD_LEAF_MIN_C
         return;
       }
       phase ^= 1u;
-      process_leaf<KMAX, uint16_t, kRec, kXl>(A, lf, s_pts, Ms, S);
+      process_leaf<kNT, uint16_t, kRec, kXl>(A, lf, s_pts, Ms, S);
     } else {
       LeafMem Mg;
-      carve<uint32_t>(A.big_scratch + (size_t)lf.start * A.big_bpp, lf.count, KMAX, &Mg);
+      carve<uint32_t>(A.big_scratch + (size_t)lf.start * A.big_bpp, lf.count, A.kmax, kNT, &Mg);
       Mg.pend = Ms.pend;  // the per-query parked keys live in shared memory on this path too
-      process_leaf<KMAX, uint32_t, kRec, kXl>(A, lf, A.spts + lf.start, Mg, S);
+      process_leaf<kNT, uint32_t, kRec, kXl>(A, lf, A.spts + lf.start, Mg, S);
     }
     __syncthreads();
   }
 }
 
-template <int KMAX, bool kRec, bool kXl>
+template <int kNT, bool kRec, bool kXl>
 inline int launch_k(const LeafArgs &a, int num_sms, cudaStream_t st) {
-  const size_t smem = leaf_smem_bytes(a.lmax, KMAX);
+  const size_t smem = leaf_smem_bytes(a.lmax, a.kmax, kNT);
   // per call (function attributes are per device, and calls may come from several threads)
-  if (cudaFuncSetAttribute(k_leaf<KMAX, kRec, kXl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+  if (cudaFuncSetAttribute(k_leaf<kNT, kRec, kXl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return -1;
-  cudaFuncSetAttribute(k_leaf<KMAX, kRec, kXl>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  cudaFuncSetAttribute(k_leaf<kNT, kRec, kXl>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        (int)cudaSharedmemCarveoutMaxShared);
-  const int nt = (a.threads == 64) ? 64 : kLeafThreads;
+  const int nt = (a.threads == 64) ? 64 : kNT;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leaf<KMAX, kRec, kXl>, nt, smem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leaf<kNT, kRec, kXl>, nt, smem) != cudaSuccess ||
       per_sm < 1)
     return -1;
   if (a.ctas_per_sm > 0 && (int)a.ctas_per_sm < per_sm) per_sm = (int)a.ctas_per_sm;
   LeafArgs la = a;
   if (la.spin_limit == 0) la.spin_limit = kSpinLimit;
-  if (launch_pdl(k_leaf<KMAX, kRec, kXl>, num_sms * per_sm, nt, smem, st, la) != cudaSuccess) return -1;
+  if (launch_pdl(k_leaf<kNT, kRec, kXl>, num_sms * per_sm, nt, smem, st, la) != cudaSuccess) return -1;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 template <bool kRec, bool kXl>
-inline int launch_kmax(const LeafArgs &a, int num_sms, cudaStream_t st) {
-  switch (leaf_kmax(a.p.k)) {
-    case 8: return launch_k<8, kRec, kXl>(a, num_sms, st);
-    case 16: return launch_k<16, kRec, kXl>(a, num_sms, st);
-    case 32: return launch_k<32, kRec, kXl>(a, num_sms, st);
-    default: return launch_k<64, kRec, kXl>(a, num_sms, st);
+inline int launch_threads(const LeafArgs &a, int num_sms, cudaStream_t st) {
+  switch (a.threads) {
+    case 256: return launch_k<256, kRec, kXl>(a, num_sms, st);
+    case 512: return launch_k<512, kRec, kXl>(a, num_sms, st);
+    default: return launch_k<128, kRec, kXl>(a, num_sms, st);
   }
 }
 

@@ -7,7 +7,7 @@
 namespace gd {
 
 int launch_leaf_xl(const LeafArgs &a, int num_sms, cudaStream_t st) {
-  return (a.use_dbg || a.use_train) ? launch_kmax<true, true>(a, num_sms, st) : launch_kmax<false, true>(a, num_sms, st);
+  return (a.use_dbg || a.use_train) ? launch_threads<true, true>(a, num_sms, st) : launch_threads<false, true>(a, num_sms, st);
 }
 
 }  // namespace gd

@@ -185,7 +185,8 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
   la.stage = stage;
   la.big_scratch = b + kOffSpill;
   la.big_bpp = leaf_big_bpp(64);
-  la.lmax = leaf_pick_lmax(p->leaf_capacity, leaf_kmax(p->k), su.smem_optin - 2048);
+  la.kmax = leaf_kmax(p->k);
+  la.lmax = leaf_pick_lmax(p->leaf_capacity, la.kmax, su.smem_optin - 2048);
   if (launch_leaf_prep(la, su.num_sms, st, nullptr) || launch_leaf(la, su.num_sms, st, nullptr)) return fail_cuda();
 
   uint32_t status = 0;
