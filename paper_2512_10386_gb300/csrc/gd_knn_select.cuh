@@ -193,10 +193,12 @@ __host__ __device__ __forceinline__ SelLevel sel_refine(const SelLevel &L, const
   return n;
 }
 
-// Does bucket B's range fit a packed key with `pbits` position bits?
+// Does bucket B's range fit a packed key with `pbits` position bits?  Every offset
+// must stay below the offset field of the padding key 0xFFFFFFFF, or a member at
+// the very top of the range would tie with the padding.
 __host__ __device__ __forceinline__ bool sel_fits(const SelCut &cut, uint32_t pbits) {
   const uint32_t range = (uint32_t)(cut.hi - (cut.lo + 1));  // largest offset in the range
-  return pbits >= 32u ? range == 0u : (uint64_t)range < (1ull << (32u - pbits));
+  return pbits >= 32u ? range == 0u : (uint64_t)range < (1ull << (32u - pbits)) - 1ull;
 }
 
 }  // namespace gd
