@@ -288,6 +288,12 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   const int kmax = leaf_kmax(p.k);
   la.kmax = kmax;
   la.lmax = leaf_pick_lmax(p.leaf_capacity, kmax, c->smem_optin - 2048);
+  if (const uint32_t above = big_leaf_above(p, n, dbg != nullptr || c->training != 0)) {
+    la.skip_big = 1;
+    la.unit_start = c->d_vals[0];  // free after the front end, as the other key buffer
+    la.far_queue = reinterpret_cast<uint2 *>(c->d_keys[front_sorted_buffer((int)p.max_depth, false) ^ 1]);
+    if (la.lmax > above) la.lmax = above;
+  }
   if (c->leaf_smem_points) {
     uint32_t l = 64;
     while (l * 2 <= c->leaf_smem_points) l *= 2;

@@ -91,6 +91,9 @@ struct Counters {
   uint32_t split_leaf;                   // first index of the largest-first order with leaves of <= kSmallLeaf points
   uint32_t xleaf_work;                   // cross-leaf kNN work counter
   uint32_t x_units;                      // cross-leaf kNN work units (leaf, 32 queries)
+  uint32_t big_units;                    // units of 1,024 points of the big leaves (gd_big.cu)
+  uint32_t big_work;                     // big-leaf kNN work counter
+  uint32_t far_count;                    // queries left to a warp of their own (gd_boxknn.cuh)
   uint32_t tile_work[kMaxPasses];        // radix-pass tile counters
   uint32_t cls_count[kLeafClasses];      // leaves per size class
   uint32_t cls_cursor[kLeafClasses];     // fill cursors of the class-ordered leaf list
@@ -202,6 +205,9 @@ struct LeafArgs {
   int use_train;
   uint32_t ctas_per_sm;         // 0 = occupancy limit
   uint32_t threads;             // threads per leaf CTA: 64, 128, 256 or 512 (0 = 128)
+  uint32_t skip_big;            // 1: leaves above lmax run in gd_big.cu's kernels, not in the fused one
+  uint32_t *unit_start;         // [n_leaves] scratch of those kernels
+  uint2 *far_queue;             // [n] likewise: (leaf of the order, query)
   int kmax;                     // leaf_kmax(p.k): rows of a spilled leaf's neighbour table
   uint32_t spin_limit;          // iterations of the bounded bulk-copy wait (0 = kSpinLimit)
   uint32_t part;                // leaves taken from the order: 0 all, 1 those before split_leaf, 2 the rest
@@ -247,6 +253,9 @@ int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launc
 // kSmallLeaf-point layout), joined back into `st`; without, one launch takes every leaf.
 int launch_leaf(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches, cudaStream_t side = nullptr,
                 cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
+// The leaf size above which a call's leaves are taken by gd_big.cu's kernels (0: none).
+uint32_t big_leaf_above(const denoise_params &p, uint32_t n, bool rec);
+int launch_big(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches);
 // the recording instantiation (debug / training outputs), in its own translation unit
 int launch_leaf_rec(const LeafArgs &a, int num_sms, cudaStream_t st);
 int launch_leaf_xl(const LeafArgs &a, int num_sms, cudaStream_t st);

@@ -76,9 +76,9 @@ __host__ __device__ __forceinline__ void sel_csa(uint32_t &h, uint32_t &l, uint3
 
 // Add 16 one-hot words into the bit-sliced counters c[0..P) (Harley-Seal tree:
 // planes 1, 2, 4, 8 through carry-save adders, the carry of weight 16 rippled
-// into the planes above).
+// into the planes above).  Returns the carry out of the last plane.
 template <int P>
-__host__ __device__ __forceinline__ void sel_add16(uint32_t (&c)[P], const uint32_t *m) {
+__host__ __device__ __forceinline__ uint32_t sel_add16(uint32_t (&c)[P], const uint32_t *m) {
   uint32_t tA, tB, fA, fB, eA, eB, s;
   sel_csa(tA, c[0], c[0], m[0], m[1]);
   sel_csa(tB, c[0], c[0], m[2], m[3]);
@@ -101,6 +101,7 @@ __host__ __device__ __forceinline__ void sel_add16(uint32_t (&c)[P], const uint3
     c[p] ^= s;
     s = t;
   }
+  return s;
 }
 
 // sum of the counts of the buckets selected by `mask`

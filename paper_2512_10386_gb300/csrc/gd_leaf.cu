@@ -53,7 +53,7 @@ __device__ __forceinline__ uint32_t class_slot(uint32_t *ctr, uint32_t cls, uint
 
 __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__restrict__ spts, Leaf *leaves,
                                                             const FrameInfo *__restrict__ frames,
-                                                            Counters *ctr, float beta, uint32_t lmax) {
+                                                            Counters *ctr, float beta, uint32_t lmax, bool skip_big) {
   __shared__ float s_ext[kPrepLeaves][3];
   pdl_wait();
   if (ctr->status & kStFatal) return;
@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__rest
       const uint32_t slot = w * kPerWarp + t, li = g + slot;
       if (li >= nl) break;
       const uint32_t start = leaves[li].start, cnt = leaves[li].count;
+      if (skip_big && cnt > lmax) continue;  // its own kernels take its box (gd_big.cu)
       float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
       for (uint32_t i0 = lane; i0 < cnt; i0 += 128) {  // four loads in flight per lane
         float4 p[4];
@@ -100,16 +101,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__rest
     if (w == 0 && g + lane < nl) {
       const uint32_t li = g + lane;
       (void)class_slot(ctr->cls_count, leaf_class(leaves[li].count, lmax), active);
-      const float delta = frames[leaves[li].frame].delta;
-      double H[3];
-      for (int a = 0; a < 3; ++a) {
-        float e = s_ext[lane][a];
-        if (e < delta) e = delta;
-        H[a] = (double)e;
-      }
-      const double V = __dmul_rn(__dmul_rn(H[0], H[1]), H[2]);
-      const double u = __ddiv_rn(V, (double)leaves[li].count);
-      leaves[li].h = __double2float_rn(__dmul_rn((double)beta, cbrt_spec(u)));
+      if (!(skip_big && leaves[li].count > lmax))
+        leaves[li].h = leaf_voxel_size(s_ext[lane], frames[leaves[li].frame].delta, leaves[li].count, beta);
     }
     __syncthreads();
   }
@@ -186,7 +179,7 @@ uint32_t leaf_pick_lmax(uint32_t leaf_capacity, int kmax, size_t smem_limit) {
 
 int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches) {
   launch_pdl(k_leaf_prep, num_sms * 4, kPrepThreads, 0, st, a.spts, const_cast<Leaf *>(a.leaves), a.frames, a.ctr, a.p.beta,
-                                                   a.lmax);
+             a.lmax, a.skip_big != 0);
   launch_pdl(k_leaf_order, num_sms * 2, 256, 0, st, a.leaves, a.ctr, a.order, a.lmax);
   if (launches) *launches += 2;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -217,6 +210,19 @@ static uint32_t leaf_auto_threads(uint32_t n, uint32_t lmax) {
 int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launches, cudaStream_t side, cudaEvent_t fork,
                 cudaEvent_t join) {
   LeafArgs a = args;
+  if (a.skip_big) {
+    // the big leaves' kernels on `st`; the other leaves, which need nothing of
+    // theirs, beside them on the side stream where there is one
+    const bool beside = side && fork && join;
+    if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a.n, a.lmax);
+    if (launches) ++*launches;
+    if (beside && (cudaEventRecord(fork, st) != cudaSuccess || cudaStreamWaitEvent(side, fork, 0) != cudaSuccess))
+      return -1;
+    if (launch_big(a, num_sms, st, launches) || launch_threads<false, false>(a, num_sms, beside ? side : st)) return -1;
+    if (beside && (cudaEventRecord(join, side) != cudaSuccess || cudaStreamWaitEvent(st, join, 0) != cudaSuccess))
+      return -1;
+    return 0;
+  }
   if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a.n, a.lmax);
   if (a.xphase != 0) {  // the cross-leaf phases: their own instantiation
     if (launches) ++*launches;

@@ -162,6 +162,22 @@ __device__ __forceinline__ uint32_t vox_index(float x, float lo, float h) {
   return (f < 2097151.0f) ? (uint32_t)f : kQMax;
 }
 
+// Eq. 12: the voxel of a point in its leaf's grid
+__device__ __forceinline__ unsigned long long voxel_key(const float4 &p, const float *lo, float h) {
+  return ((unsigned long long)vox_index(p.x, lo[0], h) << 42) | ((unsigned long long)vox_index(p.y, lo[1], h) << 21) |
+         (unsigned long long)vox_index(p.z, lo[2], h);
+}
+
+// Eq. 10-11: h = f32(beta * cbrt_spec(V_t / N_t)) from the FP32 extents, floored at
+// delta, with V_t in FP64
+__device__ __forceinline__ float leaf_voxel_size(const float *ext, float delta, uint32_t count, float beta) {
+  double H[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) H[a] = (double)(ext[a] < delta ? delta : ext[a]);
+  const double V = __dmul_rn(__dmul_rn(H[0], H[1]), H[2]);
+  return __double2float_rn(__dmul_rn((double)beta, cbrt_spec(__ddiv_rn(V, (double)count))));
+}
+
 __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
   x ^= x >> 33;
   x *= 0xff51afd7ed558ccdull;
@@ -459,6 +475,11 @@ static __device__ __noinline__ float leaf_lref(float ra, float rb, uint32_t m, u
   return __fsub_rn(lr, corr);
 }
 
+// ell_i = log2(rho_i / sqrt(rho_med^2 + eps_rho)) of a point with r_K^2 = r2
+__device__ __forceinline__ float score_ell(float r2, float r2ref, float Lref) {
+  return __fsub_rn(Lref, __fmul_rn(1.5f, log2f(__fdiv_rn(r2, r2ref))));
+}
+
 // (d^2)^(gamma/2) for gamma != 2 (the score's common case gamma = 2 needs none): out of line
 static __device__ __noinline__ float pow_half_gamma(float d2, float hg) { return exp2f(__fmul_rn(hg, log2f(d2))); }
 
@@ -525,7 +546,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
     M.hcnt[i] = 0;
   }
   __syncthreads();
-  const float lo0 = S.lo[0], lo1 = S.lo[1], lo2 = S.lo[2], h = S.h;
+  const float lo[3] = {S.lo[0], S.lo[1], S.lo[2]}, h = S.h;
   // each point's hash slot, for the gate below (wa is idle until the score weights)
   uint32_t *const vslot = reinterpret_cast<uint32_t *>(M.wa);
   for (uint32_t base = 0; base < nt && a1_on; base += NT) {
@@ -533,8 +554,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
     unsigned long long key = kInvalid;
     if (i < nt) {
       const float4 p = pts[i];
-      key = ((unsigned long long)vox_index(p.x, lo0, h) << 42) |
-            ((unsigned long long)vox_index(p.y, lo1, h) << 21) | (unsigned long long)vox_index(p.z, lo2, h);
+      key = voxel_key(p, lo, h);
     }
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, key);
     uint32_t sl = 0;
@@ -1063,8 +1083,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
     const float r2ref = S.r2ref, Lref = S.Lref;
     const float half_alpha = __fmul_rn(0.5f, P.alpha);
     for (uint32_t i = tid; i < n1; i += NT) {
-      const float r2 = M.r2[i];
-      const float ell = __fsub_rn(Lref, __fmul_rn(1.5f, log2f(__fdiv_rn(r2, r2ref))));  // log2(rho_i / sqrt(rho_med^2 + eps))
+      const float ell = score_ell(M.r2[i], r2ref, Lref);
       const float wa = __fmul_rn(half_alpha, ell);
       M.wa[i] = wa;
       // shared-memory leaves: each point's (x, y, z, weight) in one 16-byte word for
@@ -1301,9 +1320,10 @@ __global__ void __launch_bounds__(kNT, leaf_min_ctas(kNT)) k_leaf(const LeafArgs
   __syncthreads();
   pdl_wait();
   // the part of the largest-first order this launch takes: every leaf, or those
-  // before the split (more than kSmallLeaf points), or from it (the small leaves)
+  // before the split (more than kSmallLeaf points), or from it (the small leaves);
+  // without the first class where those leaves have their own kernels (gd_big.cu)
   const uint32_t n_all = A.ctr->n_leaves, split = A.ctr->split_leaf;
-  const uint32_t w_lo = (A.part == 2) ? split : 0u, w_hi = (A.part == 1) ? split : n_all;
+  const uint32_t w_lo = (A.part == 2) ? split : A.skip_big ? A.ctr->cls_count[0] : 0u, w_hi = (A.part == 1) ? split : n_all;
   uint32_t *const wctr = (kXl && A.xphase == 3) ? &A.ctr->leaf_work2
                          : (A.part == 2)         ? &A.ctr->leaf_work3
                                                  : &A.ctr->leaf_work;
