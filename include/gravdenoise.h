@@ -188,8 +188,8 @@ int denoise_set_tuning(denoise_ctx *ctx, const denoise_tuning *t);
  *               bounding box (the paper's usual choice for M).
  * `metrics` is a HOST double[3].  nn_clean [n_clean] / nn_denoised
  * [n_denoised] (host or device, may be NULL) receive the per-point nearest
- * squared distances.  Every pair of points is compared (exact nearest
- * neighbours); squared distances are FP32 with the method's operation order,
+ * squared distances.  The nearest neighbours are exact (over all pairs of
+ * points); squared distances are FP32 with the method's operation order,
  * the means FP64 in a fixed order (deterministic).
  * Errors: E_INVAL (NULL argument, an empty cloud), E_CAPACITY (a cloud larger
  * than max_points), E_NONFINITE, E_TIMEOUT, E_CUDA.
@@ -210,7 +210,7 @@ int denoise_eval_metrics(denoise_ctx *ctx, const float *clean, size_t n_clean, c
  *  device; n_i [n] uint32 counts (may be NULL); params HOST double[5] =
  *  (theta_x, theta_y, theta_z, R, T) (may be NULL).
  * The neighbour test compares the FP32 squared distance (the method's
- * operation order) with R^2; every pair is compared.
+ * operation order) with R^2, over all pairs.
  * Errors: E_INVAL (NULL argument, n = 0, G or alpha not positive and finite),
  * E_CAPACITY (n > max_points), E_NONFINITE, E_TIMEOUT, E_CUDA.
  */

@@ -669,6 +669,8 @@ int denoise_eval_metrics(denoise_ctx *ctx, const float *clean, size_t n_clean, c
   const size_t stage_a = (need + 255) & ~size_t(255), stage_b = stage_a + ((12ull * na + 255) & ~size_t(255));
   const size_t total = stage_b + 12ull * nb;
   if (total > ctx->max_points * (size_t)ctx->big_bpp) return DENOISE_E_CAPACITY;
+  const size_t box_at = (total + 255) & ~size_t(255);
+  const bool boxes = evb_takes(2ull * na * nb) && box_at + evb_scratch_bytes(na, nb) <= ctx->max_points * (size_t)ctx->big_bpp;
   int rc = DENOISE_OK;
   const float *a = stage_points(clean, na, ctx->device, (float *)(ctx->d_big + stage_a), st, &rc);
   const float *b = rc ? nullptr : stage_points(denoised, nb, ctx->device, (float *)(ctx->d_big + stage_b), st, &rc);
@@ -685,6 +687,7 @@ int denoise_eval_metrics(denoise_ctx *ctx, const float *clean, size_t n_clean, c
   e.nn_denoised = nn_denoised ? (lb == Loc::kDevice ? nn_denoised : (float *)ctx->d_gin) : nullptr;
   e.out = ctx->d_grad;
   e.scratch = ctx->d_big;
+  e.box_scratch = boxes ? ctx->d_big + box_at : nullptr;
   e.ctr = ctx->d_ctr;
   e.spin_limit = ctx->wait_limit;
   if (cudaMemsetAsync(&ctx->d_ctr->status, 0, sizeof(uint32_t), st) != cudaSuccess) return cuda_fail();
@@ -712,6 +715,8 @@ int denoise_run_baseline(denoise_ctx *ctx, const float *xyz, size_t n, double G,
   const size_t need = ev_scratch_bytes(nn, 0);
   const size_t stage = (need + 255) & ~size_t(255);
   if (stage + 12ull * nn > ctx->max_points * (size_t)ctx->big_bpp) return DENOISE_E_CAPACITY;
+  const size_t box_at = (stage + 12ull * nn + 255) & ~size_t(255);
+  const bool boxes = evb_takes((uint64_t)nn * nn) && box_at + evb_scratch_bytes(nn, 0) <= ctx->max_points * (size_t)ctx->big_bpp;
   int rc = DENOISE_OK;
   const float *x = stage_points(xyz, nn, ctx->device, (float *)(ctx->d_big + stage), st, &rc);
   if (rc) return rc;
@@ -726,6 +731,7 @@ int denoise_run_baseline(denoise_ctx *ctx, const float *xyz, size_t n, double G,
   b.n_i = n_i ? (ln == Loc::kDevice ? n_i : (uint32_t *)ctx->d_gin) : nullptr;
   b.params_out = ctx->d_partials;
   b.scratch = ctx->d_big;
+  b.box_scratch = boxes ? ctx->d_big + box_at : nullptr;
   b.ctr = ctx->d_ctr;
   b.spin_limit = ctx->wait_limit;
   if (cudaMemsetAsync(&ctx->d_ctr->status, 0, sizeof(uint32_t), st) != cudaSuccess) return cuda_fail();

@@ -177,6 +177,7 @@ struct FrontArgs {
   uint32_t leaf_capacity;
   uint32_t spin_limit;      // iterations of a bounded look-back wait (0 = kSpinLimit)
   uint32_t hold_tile1;      // test hook: tile hold_tile1 - 1 of the first radix pass never publishes (0 = off)
+  bool order_only;          // stop after the radix passes (points in octree order down to the sorted bits)
   bool full_sort;           // sort by every key bit (the cross-leaf variant searches cells of any level)
 };
 
@@ -267,6 +268,7 @@ struct EvalArgs {
   float *nn_clean, *nn_denoised;  // device [na] / [nb] nearest squared distances, or null
   double *out;                    // device [3]: mse, chamfer, psnr
   unsigned char *scratch;         // ev_scratch_bytes(na, nb) bytes, 256-byte aligned
+  unsigned char *box_scratch;     // evb_scratch_bytes(na, nb) bytes, or null: every pair is compared
   Counters *ctr;
   uint32_t spin_limit;
 };
@@ -278,10 +280,19 @@ struct BaselineArgs {
   uint32_t *n_i;                  // device [n] neighbour counts (Eq. 5), or null
   double *params_out;             // device [5]: centroid x, y, z, R, T; or null
   unsigned char *scratch;         // ev_scratch_bytes(n, 0) bytes
+  unsigned char *box_scratch;     // evb_scratch_bytes(n, 0) bytes, or null: every pair is compared
   Counters *ctr;
   uint32_t spin_limit;
 };
 size_t ev_scratch_bytes(uint32_t na, uint32_t nb);
+// The same passes over boxes (gd_eval_box.cu), for clouds whose pairs are worth them.
+bool evb_takes(uint64_t pairs);
+size_t evb_scratch_bytes(uint32_t na, uint32_t nb);
+int launch_evb_nearest(unsigned char *scratch, const float *a, uint32_t na, const float *b, uint32_t nb, float *nn_a,
+                       float *nn_b, const FrameInfo **frame_a, Counters *ctr, uint32_t spin_limit, int num_sms,
+                       cudaStream_t st);
+int launch_evb_count(unsigned char *scratch, const float *xyz, uint32_t n, const float *r2_dev, uint32_t *cnt,
+                     Counters *ctr, uint32_t spin_limit, int num_sms, cudaStream_t st);
 int launch_eval_metrics(const EvalArgs &e, int num_sms, cudaStream_t st);
 int launch_baseline(const BaselineArgs &b, int num_sms, cudaStream_t st);
 

@@ -8,7 +8,8 @@
 //
 // Both need, for every query point, a reduction over every point of another
 // set (or the same set): the nearest squared distance, or the count within R.
-// Nothing is skipped: each query meets each candidate once, so the pass is
+// Large pairs of clouds are pruned by boxes (gd_eval_box.cu); in the pass here
+// nothing is skipped: each query meets each candidate once, so it is
 // bound by the FP32 pipe (d^2 = fma(dz,dz,fma(dy,dy,dx*dx)), the method's fixed
 // operation order, in packed two-lane form), not by memory.  The candidates are
 // packed as structure of arrays and staged through shared memory by TMA bulk
@@ -285,28 +286,59 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_cross(const CrossArgs A) {
 // ---------------------------------------------------------------------------
 // finishing steps
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double sum_parts(const double *p, uint32_t n, uint32_t stride) {
-  double s = 0.0;
-  for (uint32_t i = 0; i < n; ++i) s = __dadd_rn(s, p[(size_t)i * stride]);
-  return s;
+constexpr int kEvFinThreads = 256;
+constexpr uint32_t kEvMaxParts = 1024;  // of ev_red_blocks
+
+// n partials (every `stride`-th double) into shared memory; their sum in order is
+// one thread's serial chain, which must not wait for a load at every step
+__device__ __forceinline__ void stage_parts(double *s, const double *p, uint32_t n, uint32_t stride) {
+  for (uint32_t i = threadIdx.x; i < n; i += kEvFinThreads) s[i] = p[(size_t)i * stride];
+}
+__device__ __forceinline__ double sum_parts(const double *s, uint32_t n) {
+  double v = 0.0;
+  for (uint32_t i = 0; i < n; ++i) v = __dadd_rn(v, s[i]);
+  return v;
+}
+// extents of the reduced partials (min at [3 + c], max at [6 + c]), one axis a warp: warps 0..2
+__device__ __forceinline__ void extents_of(const double *red, uint32_t nbr, double *H) {
+  const uint32_t c = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  if (c >= 3) return;
+  double lo = INFINITY, hi = -INFINITY;
+  for (uint32_t b = lane; b < nbr; b += 32u) {
+    lo = fmin(lo, red[9ull * b + 3 + c]);
+    hi = fmax(hi, red[9ull * b + 6 + c]);
+  }
+  for (int o = 16; o; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
+  }
+  if (lane == 0) H[c] = __dsub_rn(hi, lo);
 }
 
-// Eq. 29-30 from the two sums and the clean cloud's extents.
-__global__ void k_ev_metrics(const double *part_a, uint32_t nba, const double *part_b, uint32_t nbb,
-                             const double *red_clean, uint32_t nbr, uint32_t na, uint32_t nb, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double mse = __ddiv_rn(sum_parts(part_a, nba, 1), (double)na);
-  const double back = __ddiv_rn(sum_parts(part_b, nbb, 1), (double)nb);
-  double M2 = 0.0;
-  for (int c = 0; c < 3; ++c) {
-    double lo = INFINITY, hi = -INFINITY;
-    for (uint32_t b = 0; b < nbr; ++b) {
-      lo = fmin(lo, red_clean[9ull * b + 3 + c]);
-      hi = fmax(hi, red_clean[9ull * b + 6 + c]);
-    }
-    const double e = __dsub_rn(hi, lo);
-    M2 = __dadd_rn(M2, __dmul_rn(e, e));
+// Eq. 29-30 from the two sums and the clean cloud's extents (from the partials, or
+// from the front end's frame where that took them).
+__global__ void __launch_bounds__(kEvFinThreads) k_ev_metrics(const double *part_a, uint32_t nba, const double *part_b,
+                                                              uint32_t nbb, const double *red_clean, uint32_t nbr,
+                                                              const FrameInfo *frame, uint32_t na, uint32_t nb,
+                                                              double *out) {
+  __shared__ double s_a[kEvMaxParts], s_b[kEvMaxParts], s_sum[2], s_h[3];
+  stage_parts(s_a, part_a, nba, 1);
+  stage_parts(s_b, part_b, nbb, 1);
+  if (frame) {
+    if (threadIdx.x < 3)
+      s_h[threadIdx.x] = __dsub_rn((double)ord2f(frame->hi_ord[threadIdx.x]), (double)ord2f(frame->lo_ord[threadIdx.x]));
+  } else {
+    extents_of(red_clean, nbr, s_h);
   }
+  __syncthreads();
+  if (threadIdx.x == 0) s_sum[0] = sum_parts(s_a, nba);
+  if (threadIdx.x == 32) s_sum[1] = sum_parts(s_b, nbb);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double mse = __ddiv_rn(s_sum[0], (double)na);
+  const double back = __ddiv_rn(s_sum[1], (double)nb);
+  double M2 = 0.0;
+  for (int c = 0; c < 3; ++c) M2 = __dadd_rn(M2, __dmul_rn(s_h[c], s_h[c]));
   out[0] = mse;
   out[1] = __dadd_rn(mse, back);
   out[2] = 10.0 * log10(M2 / mse);
@@ -314,20 +346,18 @@ __global__ void k_ev_metrics(const double *part_a, uint32_t nba, const double *p
 
 // Eq. 1-3 and 7 of the baseline: centroid, extents, R (and R^2 rounded down to
 // FP32: for a float d^2, d^2 <= R^2 exactly when d^2 <= RD(R^2)), T.
-// g[0..2] theta, g[3] R, g[4] T, g[5] bits of RD(R^2) as a double
-__global__ void k_bl_params(const double *part, uint32_t nbr, uint32_t n, double G, double alpha, double *g,
-                            float *r2f_out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double H[3];
-  for (int c = 0; c < 3; ++c) {
-    g[c] = __ddiv_rn(sum_parts(part + c, nbr, 9), (double)n);
-    double lo = INFINITY, hi = -INFINITY;
-    for (uint32_t b = 0; b < nbr; ++b) {
-      lo = fmin(lo, part[9ull * b + 3 + c]);
-      hi = fmax(hi, part[9ull * b + 6 + c]);
-    }
-    H[c] = __dsub_rn(hi, lo);
+// g[0..2] theta, g[3] R, g[4] T
+__global__ void __launch_bounds__(kEvFinThreads) k_bl_params(const double *part, uint32_t nbr, uint32_t n, double G,
+                                                             double alpha, double *g, float *r2f_out) {
+  __shared__ double s_p[3][kEvMaxParts], H[3];
+  for (int c = 0; c < 3; ++c) stage_parts(s_p[c], part + c, nbr, 9);
+  extents_of(part, nbr, H);
+  __syncthreads();
+  if ((threadIdx.x & 31u) == 0 && threadIdx.x < 96) {
+    const uint32_t c = threadIdx.x >> 5;
+    g[c] = __ddiv_rn(sum_parts(s_p[c], nbr), (double)n);
   }
+  if (threadIdx.x != 96) return;
   const double area = __dadd_rn(__dadd_rn(__dmul_rn(H[0], H[1]), __dmul_rn(H[0], H[2])), __dmul_rn(H[1], H[2]));
   const double R = __ddiv_rn(__dmul_rn(6.0, area), (double)n);
   const double T = __ddiv_rn(__dmul_rn(__dmul_rn(alpha, G), __dadd_rn(__dadd_rn(H[0], H[1]), H[2])), (double)n);
@@ -361,7 +391,7 @@ size_t ev_scratch_bytes(uint32_t na, uint32_t nb) {
 }
 
 namespace {
-inline uint32_t ev_red_blocks(uint32_t n) { return min(1024u, (n + 4095u) / 4096u + 1u); }
+inline uint32_t ev_red_blocks(uint32_t n) { return min(kEvMaxParts, (n + 4095u) / 4096u + 1u); }
 
 int launch_cross(int mode, const CrossArgs &base, int num_sms, cudaStream_t st) {
   CrossArgs a = base;
@@ -395,28 +425,39 @@ int launch_eval_metrics(const EvalArgs &e, int num_sms, cudaStream_t st) {
   const uint32_t ra = ev_red_blocks(e.na), rb = ev_red_blocks(e.nb);
   double *red = (double *)take(8ull * 9 * ra);
   double *pa_sum = (double *)take(8ull * ra), *pb_sum = (double *)take(8ull * rb);
-  const uint32_t g = (uint32_t)num_sms * 4;
-  k_ev_pack<<<g, 256, 0, st>>>(e.clean, e.na, pa, ax, ay, az, e.ctr);
-  k_ev_pack<<<g, 256, 0, st>>>(e.denoised, e.nb, pb, bx, by, bz, e.ctr);
-  k_ev_reduce<<<ra, kEvRedThreads, 0, st>>>(ax, ay, az, e.na, red);
-  CrossArgs c{};
-  c.ctr = e.ctr;
-  c.spin_limit = e.spin_limit ? e.spin_limit : kSpinLimit;
-  // clean -> denoised (Eq. 29's correspondence and Eq. 30's first term)
-  c.qx = ax; c.qy = ay; c.qz = az; c.nq = e.na;
-  c.cx = bx; c.cy = by; c.cz = bz; c.ncand = pb;
-  c.out = da;
-  if (launch_cross(0, c, num_sms, st)) return -1;
-  // denoised -> clean (Eq. 30's second term)
-  c.qx = bx; c.qy = by; c.qz = bz; c.nq = e.nb;
-  c.cx = ax; c.cy = ay; c.cz = az; c.ncand = pa;
-  c.out = db;
-  if (launch_cross(0, c, num_sms, st)) return -1;
+  const FrameInfo *frame = nullptr;
+  if (e.box_scratch) {
+    if (e.nn_clean) da = reinterpret_cast<uint32_t *>(e.nn_clean);  // the distances go where the caller wants them
+    if (e.nn_denoised) db = reinterpret_cast<uint32_t *>(e.nn_denoised);
+    if (launch_evb_nearest(e.box_scratch, e.clean, e.na, e.denoised, e.nb, reinterpret_cast<float *>(da),
+                           reinterpret_cast<float *>(db), &frame, e.ctr, e.spin_limit, num_sms, st))
+      return -1;
+  } else {
+    const uint32_t g = (uint32_t)num_sms * 4;
+    k_ev_pack<<<g, 256, 0, st>>>(e.clean, e.na, pa, ax, ay, az, e.ctr);
+    k_ev_pack<<<g, 256, 0, st>>>(e.denoised, e.nb, pb, bx, by, bz, e.ctr);
+    k_ev_reduce<<<ra, kEvRedThreads, 0, st>>>(ax, ay, az, e.na, red);
+    CrossArgs c{};
+    c.ctr = e.ctr;
+    c.spin_limit = e.spin_limit ? e.spin_limit : kSpinLimit;
+    // clean -> denoised (Eq. 29's correspondence and Eq. 30's first term)
+    c.qx = ax; c.qy = ay; c.qz = az; c.nq = e.na;
+    c.cx = bx; c.cy = by; c.cz = bz; c.ncand = pb;
+    c.out = da;
+    if (launch_cross(0, c, num_sms, st)) return -1;
+    // denoised -> clean (Eq. 30's second term)
+    c.qx = bx; c.qy = by; c.qz = bz; c.nq = e.nb;
+    c.cx = ax; c.cy = ay; c.cz = az; c.ncand = pa;
+    c.out = db;
+    if (launch_cross(0, c, num_sms, st)) return -1;
+  }
   k_ev_sum<<<ra, kEvRedThreads, 0, st>>>(da, e.na, pa_sum);
   k_ev_sum<<<rb, kEvRedThreads, 0, st>>>(db, e.nb, pb_sum);
-  k_ev_metrics<<<1, 32, 0, st>>>(pa_sum, ra, pb_sum, rb, red, ra, e.na, e.nb, e.out);
-  if (e.nn_clean) cudaMemcpyAsync(e.nn_clean, da, 4ull * e.na, cudaMemcpyDeviceToDevice, st);
-  if (e.nn_denoised) cudaMemcpyAsync(e.nn_denoised, db, 4ull * e.nb, cudaMemcpyDeviceToDevice, st);
+  k_ev_metrics<<<1, kEvFinThreads, 0, st>>>(pa_sum, ra, pb_sum, rb, red, ra, frame, e.na, e.nb, e.out);
+  if (!e.box_scratch) {
+    if (e.nn_clean) cudaMemcpyAsync(e.nn_clean, da, 4ull * e.na, cudaMemcpyDeviceToDevice, st);
+    if (e.nn_denoised) cudaMemcpyAsync(e.nn_denoised, db, 4ull * e.nb, cudaMemcpyDeviceToDevice, st);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -432,17 +473,21 @@ int launch_baseline(const BaselineArgs &b, int num_sms, cudaStream_t st) {
   float *r2f = (float *)take(16);
   k_ev_pack<<<(uint32_t)num_sms * 4, 256, 0, st>>>(b.xyz, b.n, pn, x, y, z, b.ctr);
   k_ev_reduce<<<rn, kEvRedThreads, 0, st>>>(x, y, z, b.n, red);
-  k_bl_params<<<1, 32, 0, st>>>(red, rn, b.n, b.G, b.alpha, gpar, r2f);
-  // the radius is a device value: read it into the pass's arguments on the device side
-  CrossArgs c{};
-  c.ctr = b.ctr;
-  c.spin_limit = b.spin_limit ? b.spin_limit : kSpinLimit;
-  c.qx = x; c.qy = y; c.qz = z; c.nq = b.n;
-  c.cx = x; c.cy = y; c.cz = z; c.ncand = pn;
-  c.out = cnt;
-  c.r2f = 0.0f;
-  c.r2f_dev = r2f;
-  if (launch_cross(1, c, num_sms, st)) return -1;
+  k_bl_params<<<1, kEvFinThreads, 0, st>>>(red, rn, b.n, b.G, b.alpha, gpar, r2f);
+  // the radius is a device value: the count reads it there
+  if (b.box_scratch) {
+    if (launch_evb_count(b.box_scratch, b.xyz, b.n, r2f, cnt, b.ctr, b.spin_limit, num_sms, st)) return -1;
+  } else {
+    CrossArgs c{};
+    c.ctr = b.ctr;
+    c.spin_limit = b.spin_limit ? b.spin_limit : kSpinLimit;
+    c.qx = x; c.qy = y; c.qz = z; c.nq = b.n;
+    c.cx = x; c.cy = y; c.cz = z; c.ncand = pn;
+    c.out = cnt;
+    c.r2f = 0.0f;
+    c.r2f_dev = r2f;
+    if (launch_cross(1, c, num_sms, st)) return -1;
+  }
   k_bl_decide<<<(uint32_t)num_sms * 4, 256, 0, st>>>(x, y, z, b.n, cnt, gpar, b.G, b.keep);
   if (b.params_out) cudaMemcpyAsync(b.params_out, gpar, 8ull * 5, cudaMemcpyDeviceToDevice, st);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;

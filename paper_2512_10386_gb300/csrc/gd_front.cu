@@ -829,6 +829,10 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
     launch_pdl(k_pack, a.ntiles, kFrontThreads, 0, st, a.xyz, a.tiles, a.spts, a.ctr);
     ++nl;
   }
+  if (a.order_only) {
+    if (launches) *launches += nl;
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  }
   // a capacity above any frame's size means the same as "the root is a leaf"; clamped
   // so that the finder's window arithmetic (cap + 1) cannot wrap
   const uint32_t cap = a.leaf_capacity < (1u << 30) ? a.leaf_capacity : (1u << 30);
