@@ -330,9 +330,18 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
       xa.dbg = *dbg;
       xa.use_dbg = 1;
     }
-    xa.unit_start = c->d_vals[0];  // free after the front end
+    // scratch that is free here: the sort's buffers, the half of the neighbour table
+    // (64 entries a point) that K <= 32 leaves, the spill area between the leaf phases
+    xa.unit_start = c->d_vals[0];
+    xa.masks = c->d_vals[1];
+    xa.far_queue = reinterpret_cast<uint2 *>(c->d_keys[front_sorted_buffer((int)p.max_depth, true) ^ 1]);
+    xa.boxes = reinterpret_cast<unsigned char *>(c->x_nbr + 32 * c->max_points);
+    xa.xrho = reinterpret_cast<float4 *>(c->x_nbr + 48 * c->max_points);
+    xa.slices = c->d_big;
+    xa.slice_bpp = c->big_bpp;
     if (launch_xleaf_knn(xa, c->num_sms, st, &launches)) return cuda_fail();
     la.xphase = 3;
+    la.xrho = p.k <= 32 ? xa.xrho : nullptr;
   }
   if (launch_leaf(la, c->num_sms, st, &launches, c->side_stream, c->fork_ev, c->join_ev)) return cuda_fail();
   if (use_events) cudaEventRecord(c->ev[5], st);

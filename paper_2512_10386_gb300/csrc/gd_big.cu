@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_big_knn(const LeafArgs A) {
     const BigSrc src{M.pts, n, M.box};
     float theta;
     uint32_t far;
-    if (!bk_knn(src, S, act, q, me.x, me.y, me.z, k, 0u, n, theta, far)) atomicOr(&A.ctr->status, kStInternal);
+    if (!bk_knn(src, S, act, q, me.x, me.y, me.z, k, 0u, n, bk_share(n), theta, far)) atomicOr(&A.ctr->status, kStInternal);
     const float delta = A.frames[lf.frame].delta, delta2 = __fmul_rn(delta, delta);
     const bool gone = (far >> lane) & 1u;
     if (act) M.r2[q] = (theta < delta2 && !gone) ? delta2 : theta;  // (a far query's bound, for its own warp)

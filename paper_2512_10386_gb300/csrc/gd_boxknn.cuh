@@ -30,7 +30,10 @@ constexpr int kBkLowPlanes = 11;     // rippled always; the carry above them is 
 // A chunk costs the warp about 700 instructions (count and emit), a query with a
 // warp of its own about 2,000: a query is left to its own once its share of the
 // chunks it wants (each split evenly over the queries that want it) is this many.
-constexpr float kBkShare = 4.0f;
+// With few points the last warp's time counts, and queries leave earlier.  Measured,
+// cross-leaf calls in us at shares 2 / 4 / 8 / never: 30k points 532 / 661 / 976 / 1015,
+// 100k 839 / 1050 / 1389 / 2674, 300k 1877 / 1895 / 2271 / 4893, 560k 3683 / 3009 / 3251 / 8951.
+__device__ __forceinline__ float bk_share(uint32_t n) { return n < 150000u ? 2.0f : 4.0f; }
 constexpr uint32_t kBkFarK = 32;     // its list has one entry per lane
 
 // One warp's shared memory.
@@ -50,7 +53,7 @@ struct BkShared {
 // The queries (lanes) to leave to a warp of their own.
 template <typename Src>
 __device__ __forceinline__ uint32_t bk_costly(const Src &src, const Box &qb, float qx, float qy, float qz, bool act,
-                                              float mine) {
+                                              float mine, float most) {
   const uint32_t lane = threadIdx.x & 31u;
   const Box me = box_point(qx, qy, qz);
   float share = 0.0f;
@@ -87,8 +90,8 @@ __device__ __forceinline__ uint32_t bk_costly(const Src &src, const Box &qb, flo
         const bool w = box_lower(x, me) <= want;
         const uint32_t m = __ballot_sync(0xFFFFFFFFu, w);
         if (w) share += rcp_hw((float)__popc(m));
-        if (__any_sync(0xFFFFFFFFu, share >= kBkShare && want >= 0.0f)) {
-          if (share >= kBkShare) want = -1.0f;
+        if (__any_sync(0xFFFFFFFFu, share >= most && want >= 0.0f)) {
+          if (share >= most) want = -1.0f;
           bound = ord2f(__reduce_max_sync(0xFFFFFFFFu, f2ord(want)));
           if (bound < 0.0f) return __ballot_sync(0xFFFFFFFFu, act);
         }
@@ -345,13 +348,14 @@ __device__ __forceinline__ void bk_knn_far(const Src &src, uint32_t q, float qx,
 // The k nearest of the lane's query (qx, qy, qz) at position q (a lane without a
 // query shadows another lane's, act = false) into S.row[lane][0..k), ascending
 // positions.  [w0, w1) is the range of positions around q to take theta_0 from
-// (all of them candidates or NaN), near0 .. near1 the chunks of the near count.
+// (all of them candidates or NaN), `share` what makes a query costly.
 // theta receives the k-th squared distance; `far` the lanes whose queries are left
 // to a warp of their own (none where k > kBkFarK), theta then a bound of it.
 // Returns false if the passes disagree (cannot happen).
 template <typename Src, int KROW>
 __device__ __forceinline__ bool bk_knn(const Src &src, BkShared<KROW> &S, bool act, uint32_t q, float qx, float qy,
-                                       float qz, uint32_t k, uint32_t w0, uint32_t w1, float &theta, uint32_t &far) {
+                                       float qz, uint32_t k, uint32_t w0, uint32_t w1, float share,
+                                       float &theta, uint32_t &far) {
   const uint32_t lane = threadIdx.x & 31u;
   f32x2 QX = pk2(qx, qx), QY = pk2(qy, qy), QZ = pk2(qz, qz);
   Box qb = box_warp_union(box_point(qx, qy, qz));
@@ -410,7 +414,7 @@ __device__ __forceinline__ bool bk_knn(const Src &src, BkShared<KROW> &S, bool a
   }
   float far_bound = 0.0f;
   if (KROW <= (int)kBkFarK) {
-    far = bk_costly(src, qb, qx, qy, qz, act, __int_as_float(L.tb));
+    far = bk_costly(src, qb, qx, qy, qz, act, __int_as_float(L.tb), share);
     if (far) {  // they shadow one of the queries that stay
       const uint32_t stay = __ballot_sync(0xFFFFFFFFu, act) & ~far;
       const bool gone = (far >> lane) & 1u;

@@ -219,6 +219,7 @@ struct LeafArgs {
   const uint32_t *xnbr;         // [n][k] neighbours (sorted positions), by sorted position
   const float *xr2;             // [n] floored r_K^2 by sorted position
   const uint32_t *xkeff;        // [n] k_eff by sorted position (0: no neighbour)
+  const float4 *xrho;           // [n] point and log2 of its density by sorted position (K <= 32, else null)
 };
 
 // Cross-leaf kNN (gd_xleaf.cu): for the P_1 points of every leaf, the k_eff
@@ -237,6 +238,12 @@ struct XleafArgs {
   float *xr2;
   uint32_t *xkeff;
   uint32_t *unit_start;  // [n_leaves] scratch: first work unit of each leaf (K <= 32)
+  unsigned char *boxes;  // scratch: box_bytes(n) bytes, 32-byte aligned (K <= 32)
+  uint32_t *masks;       // scratch: [ceil(n / 32)]
+  float4 *xrho;          // [n] (x, y, z, log2 density) by sorted position (K <= 32)
+  uint2 *far_queue;      // scratch: [n]
+  unsigned char *slices; // the spill area: each leaf's ranges at the start of its slice
+  uint32_t slice_bpp;
   denoise_debug dbg;
   int use_dbg;
 };

@@ -475,6 +475,11 @@ static __device__ __noinline__ float leaf_lref(float ra, float rb, uint32_t m, u
   return __fsub_rn(lr, corr);
 }
 
+// log2(rho) = log2(k_eff) - log2(4/3 pi) - 1.5 log2(r2)
+__device__ __forceinline__ float log2_density(uint32_t keff, float r2) {
+  return __fsub_rn(__fsub_rn(log2f((float)keff), 2.0665336287511624f), __fmul_rn(1.5f, log2f(r2)));
+}
+
 // ell_i = log2(rho_i / sqrt(rho_med^2 + eps_rho)) of a point with r_K^2 = r2
 __device__ __forceinline__ float score_ell(float r2, float r2ref, float Lref) {
   return __fsub_rn(Lref, __fmul_rn(1.5f, log2f(__fdiv_rn(r2, r2ref))));
@@ -1164,10 +1169,16 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
 #pragma unroll 1
         for (uint32_t t = 0; t < keff; ++t) {
           const uint32_t j = nl[t];
-          const float4 pj = A.spts[j];
+          float4 pj;
+          float lj;
+          if (A.xrho) {  // K <= 32: the search left log2(rho_j) beside the point
+            pj = A.xrho[j];
+            lj = pj.w;
+          } else {
+            pj = A.spts[j];
+            lj = log2_density(A.xkeff[j], A.xr2[j]);
+          }
           const float d2 = sqdist(xi, yi, zi, pj.x, pj.y, pj.z);
-          const float lj = __fsub_rn(__fsub_rn(log2f((float)A.xkeff[j]), 2.0665336287511624f),
-                                     __fmul_rn(1.5f, log2f(A.xr2[j])));
           const float waj = __fmul_rn(half_alpha, __fsub_rn(lj, lsh));
           const float wt = ex2_hw(__fmaf_rn(-d2, ci, __fadd_rn(ai, waj)));
           const float D = g2 ? d2 : pow_half_gamma(d2, hg);

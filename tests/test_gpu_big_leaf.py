@@ -84,3 +84,36 @@ def test_batch_of_one_leaf_frames_and_small_leaves():
         offs.append(offs[-1] + len(p))
     _check(torch.cat(parts), offs, k=8, leaf_capacity=ONE)
     _check(torch.cat(parts), offs, k=8, leaf_capacity=1100)
+
+
+@pytest.mark.parametrize("n,cap,k,kw", [
+    (3000, 512, 12, {}), (20_000, 256, 32, {}), (20_000, 64, 1, {}), (5000, ONE, 24, {}), (9000, 30, 20, {}),
+    (9000, 128, 32, {"max_depth": 2}), (4000, 512, 16, {"min_vox_count": 40}), (1, 512, 8, {}), (33, 8, 32, {}),
+])
+@pytest.mark.parametrize("make", ["surface", "lattice", "dups"])
+def test_cross_leaf_box_search_against_the_lists(n, cap, k, kw, make):
+    """Cross-leaf neighbours of the box search (K <= 32) against the exhaustive lists, which
+    K = 33 takes: the first K of the 33 in (d^2, input index) order are the K nearest."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2512_10386_gb300 import Denoiser, Params
+    if make == "surface":
+        xyz = _surface(n, n + k)
+    elif make == "lattice":
+        xyz = _lattice(max(2, round(n ** (1 / 3))), 0.125)
+    else:
+        xyz = _dups(n, max(1, n // 9))
+    xyz = xyz.cuda().contiguous()
+    d = Denoiser(max_points=len(xyz))
+    try:
+        d.set_cross_leaf(True)
+        kw = {"leaf_capacity": cap, "cross_leaf": 1, "min_vox_count": 2, **kw}
+        a = d.run_debug(xyz, Params(k=k, **kw))
+        b = d.run_debug(xyz, Params(k=33, **kw))
+        p1 = b["stage"] != 1
+        assert torch.equal(a["nbr"][p1], b["nbr"][p1][:, :k])
+        assert torch.equal(a["nbr_d2"][p1], b["nbr_d2"][p1][:, :k])
+        r = d.run(xyz, Params(k=k, **kw))
+        assert torch.equal(r.mask, a["mask"]) and torch.equal(r.score, a["score"])
+    finally:
+        d.close()
