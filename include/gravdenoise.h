@@ -98,7 +98,7 @@ typedef struct denoise_ctx denoise_ctx;
  * per-leaf spill space) is allocated here, sized for max_points; the forward
  * calls (denoise_run, denoise_run_batch, denoise_run_debug) allocate no device
  * memory.  Two optional features allocate later, on request: the training
- * cache, made by the first denoise_set_training(ctx, 1) (about 520 bytes a
+ * cache, made by the first denoise_set_training(ctx, 1) (about 37 bytes a
  * point), and the cross-leaf kNN tables, made by the first
  * denoise_set_cross_leaf(ctx, 1) (about 265 bytes a point); the metric and
  * baseline calls use the context's scratch and allocate nothing.  The largest buffer
@@ -281,7 +281,7 @@ int denoise_run_debug(denoise_ctx *ctx, const float *xyz, size_t n, const denois
 /*
  * Differentiable form (reading of Sec. 3 for calibration; the paper itself
  * only thresholds).  With training enabled, the forward keeps, for every
- * scored point, its neighbour list and density terms on the device.
+ * scored point, the sums over its neighbours that the backward needs.
  *  denoise_soft_removal: removal probability r_i = 1 - sigmoid((ln F_i - tau)/T)
  *    for points of P_2 and 1 for points removed by the gates, for the last
  *    forward call and its parameters; removal [n] float32 (host or device).

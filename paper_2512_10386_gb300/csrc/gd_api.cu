@@ -155,7 +155,7 @@ void free_ctx(denoise_ctx *c) {
   void *dptrs[] = {c->d_xyz, c->d_mask, c->d_score, c->d_stage, c->d_gin, c->d_keys[0], c->d_keys[1],
                    c->d_vals[0], c->d_vals[1], c->d_spts, c->d_frames, c->d_tiles, c->d_hist, c->d_base,
                    c->d_lookback, c->d_leaves, c->d_order, c->d_ctr, c->d_big, c->d_partials, c->d_grad,
-                   c->train.nbr, c->train.nd2, c->train.ell, c->train.r2, c->train.F, c->train.stage,
+                   c->train.sums, c->train.ell, c->train.r2, c->train.F, c->train.stage,
                    c->x_nbr, c->x_r2, c->x_keff, c->x_flag};
   for (void *p : dptrs)
     if (p) cudaFree(p);
@@ -301,7 +301,6 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   }
   if (c->training) {
     la.train = c->train;
-    la.train.k = p.k;
     la.use_train = 1;
   }
   if (launch_leaf_prep(la, c->num_sms, st, &launches)) return cuda_fail();
@@ -798,8 +797,7 @@ int denoise_set_training(denoise_ctx *ctx, int enable) {
     if (cudaSetDevice(ctx->device) != cudaSuccess) return DENOISE_E_CUDA;
     const size_t N = ctx->max_points;
     int e = 0;
-    e |= dalloc(&ctx->train.nbr, N * 64);
-    e |= dalloc(&ctx->train.nd2, N * 64);
+    e |= dalloc(&ctx->train.sums, N * 3);
     e |= dalloc(&ctx->train.ell, N);
     e |= dalloc(&ctx->train.r2, N);
     e |= dalloc(&ctx->train.F, N);
@@ -849,7 +847,6 @@ int denoise_soft_removal(denoise_ctx *ctx, float *removal, void *stream) {
   const bool dev = lr == Loc::kDevice;
   BackArgs a{};
   a.train = ctx->train;
-  a.train.k = ctx->last_p.k;
   a.n = (uint32_t)ctx->last_n;
   a.p = ctx->last_p;
   a.removal = dev ? removal : ctx->d_score;
@@ -869,7 +866,6 @@ int denoise_backward(denoise_ctx *ctx, const float *grad_removal, double *grad4,
   cudaStream_t st = (cudaStream_t)stream;
   BackArgs a{};
   a.train = ctx->train;
-  a.train.k = ctx->last_p.k;
   a.n = (uint32_t)ctx->last_n;
   a.p = ctx->last_p;
   if (a.n == 0) {

@@ -103,15 +103,14 @@ struct Counters {
   unsigned long long score_terms;        // neighbour terms summed by the score (Eq. 21)
 };
 
-// Train-mode cache written by the forward for the backward.
+// Train-mode cache written by the forward for the backward, by input index.
 struct TrainCache {
-  uint32_t *nbr;    // [n][k] neighbour global indices (P_1 points), 0xFFFFFFFF pad
-  float *nd2;       // [n][k] squared neighbour distances (FP32), 0 pad
+  double *sums;     // [n][3] over a scored point's neighbour terms t: sum t ln(W), sum t d^2,
+                    //        sum t (d^2)^(gamma/2) ln(d^2) / ((d^2)^(gamma/2) + eps_k)
   float *ell;       // [n] log2(rho_i / sqrt(rho_med^2 + eps_rho)) for P_1 points
-  float *r2;        // [n] floored r_K^2 for P_1 points
+  float *r2;        // [n] floored r_K^2 of scored points
   float *F;         // [n] score (P_2), 0 otherwise
   uint8_t *stage;   // [n]
-  uint32_t k;
 };
 
 __device__ __forceinline__ uint32_t f2ord(float f) {

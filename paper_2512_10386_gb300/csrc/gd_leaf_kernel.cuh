@@ -498,6 +498,49 @@ __device__ __forceinline__ bool rec_index_ok(const LeafArgs &A, uint32_t g) {
   return false;
 }
 
+// The sums over a scored point's neighbour terms that the backward pass needs
+// (TrainCache), taken where the neighbours are at hand: keeping the neighbour lists
+// for the backward instead meant 256 scattered bytes a point written and read again.
+// Each sum is an unevaluated pair of floats: products split exactly by a fused
+// multiply-add, additions with their exact rounding error, so it carries what a
+// double-precision sum of the FP32 factors' products does, at FP32 rate.
+struct PairSum {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
+    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
+    hi = t;
+    lo = __fadd_rn(lo, __fadd_rn(err, e));
+  }
+  __device__ __forceinline__ double value() const { return __dadd_rn((double)hi, (double)lo); }
+};
+struct TrainSums {
+  PairSum w, d, g;
+  __device__ __forceinline__ void add(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
+    const float lw2 = __fadd_rn(elli, ellj);  // log2 W_ij
+    const float D = g2 ? d2 : exp2f(0.5f * P.gamma * log2f(d2));
+    const float q = __fadd_rn(D, P.eps_k);
+    const float t = __fdiv_rn(exp2f(__fmaf_rn(__fmul_rn(0.5f, P.alpha), lw2, -__fmul_rn(d2, ci))), q);
+    if (t == 0.0f) return;  // (a neighbour of density 0 has ln W = -infinity)
+    w.add(t, __fmul_rn(lw2, 0.6931471805599453f));  // ln W_ij
+    d.add(t, d2);
+    if (d2 > 0.0f) {  // D / q = 1 - eps_k / q
+      const float l = logf(d2);
+      g.add(t, l);
+      if (P.eps_k > 0.0f) g.add(__fmul_rn(t, -__fdiv_rn(P.eps_k, q)), l);
+    }
+  }
+  __device__ __forceinline__ void store(const LeafArgs &A, uint32_t i, float r2) const {
+    if (!rec_index_ok(A, i)) return;
+    double *const s = A.train.sums + 3ull * i;
+    s[0] = w.value();
+    s[1] = d.value();
+    s[2] = g.value();
+    A.train.r2[i] = r2;
+  }
+};
+
 template <bool kRec>
 __device__ __forceinline__ void write_point(const LeafArgs &A, uint32_t g, uint8_t mk, float sc, uint8_t st) {
   if (g >= A.n) {  // cannot happen with a consistent sort; never write out of bounds
@@ -800,16 +843,12 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         }
       };
       // Record neighbour t (position npos, input index g, distance d2) where the
-      // table keeps positions (global path) and in the debug / training outputs.
+      // table keeps positions (global path) and in the debug outputs.
       auto emit = [&](uint32_t t, uint32_t npos, uint32_t g, float d2) {
         if constexpr (!kPacked) nbr[(size_t)t * cap + qq] = (IdxT)npos;
-        if (kRec && (dbg_n || dbg_d || A.use_train) && rec_index_ok(A, gq)) {
+        if (kRec && (dbg_n || dbg_d) && rec_index_ok(A, gq)) {
           if (dbg_n) A.dbg.nbr[(size_t)gq * P.k + t] = g;
           if (dbg_d) A.dbg.nbr_d2[(size_t)gq * P.k + t] = d2;
-          if (A.use_train) {
-            A.train.nbr[(size_t)gq * P.k + t] = g;
-            A.train.nd2[(size_t)gq * P.k + t] = d2;
-          }
         }
       };
       // pass 2, by chunks of 32 candidates: two bit masks (d^2 <= bottom of B's
@@ -857,6 +896,7 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
           cm |= (em ? 1u : 0u) << ((c0 >> 5) & 31u);
         }
         if constexpr (!kPacked || kRec) {
+          if (kPacked && !dbg_n && !dbg_d) em = 0;  // training alone records no list
           while (em) {
             const uint32_t ju = c0 + (uint32_t)(__ffs(em) - 1);
             em &= em - 1u;
@@ -963,17 +1003,12 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         const float rt = (theta < delta2) ? delta2 : theta;
         M.r2[qq] = rt;
         if (kPacked && use_cm) M.cmask[qq] = cm;
-        if (kRec && (A.use_dbg || A.use_train) && rec_index_ok(A, gq)) {
+        if (kRec && A.use_dbg && rec_index_ok(A, gq)) {
           for (uint32_t t = keff; t < P.k; ++t) {
             if (dbg_n) A.dbg.nbr[(size_t)gq * P.k + t] = 0xFFFFFFFFu;
             if (dbg_d) A.dbg.nbr_d2[(size_t)gq * P.k + t] = 0.0f;
-            if (A.use_train) {
-              A.train.nbr[(size_t)gq * P.k + t] = 0xFFFFFFFFu;
-              A.train.nd2[(size_t)gq * P.k + t] = 0.0f;
-            }
           }
-          if (A.use_dbg && A.dbg.r2) A.dbg.r2[gq] = rt;
-          if (A.use_train) A.train.r2[gq] = rt;
+          if (A.dbg.r2) A.dbg.r2[gq] = rt;
         }
       }
       uint32_t nb = 0;
@@ -1090,7 +1125,8 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
     for (uint32_t i = tid; i < n1; i += NT) {
       const float ell = score_ell(M.r2[i], r2ref, Lref);
       const float wa = __fmul_rn(half_alpha, ell);
-      M.wa[i] = wa;
+      // (training: ell itself, which the gradient sums need; the score's weight is in the word below)
+      M.wa[i] = (kRec && kPacked && A.use_train) ? ell : wa;
       // shared-memory leaves: each point's (x, y, z, weight) in one 16-byte word for
       // the score's neighbour reads (region R is idle between the median and Top-lambda)
       if constexpr (kPacked) reinterpret_cast<float4 *>(M.sbuf)[i] = make_float4(X[i], Y[i], Z[i], wa);
@@ -1111,7 +1147,12 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
     for (uint32_t i = tid; i < n1; i += NT) {
       if (!M.flag[i]) continue;
       const float xi = X[i], yi = Y[i], zi = Z[i];
-      const float ai = M.wa[i], ci = __fdiv_rn(c2, M.r2[i]);  // r2_i's last read: F_i takes its place
+      const bool train = kRec && A.use_train;
+      const float r2i = M.r2[i], ci = __fdiv_rn(c2, r2i);  // r2_i's last read: F_i takes its place
+      const float ai = (train && kPacked) ? __fmul_rn(__fmul_rn(0.5f, P.alpha), M.wa[i]) : M.wa[i];
+      float elli = 0.0f;
+      TrainSums ts;
+      if (train) elli = kPacked ? M.wa[i] : (W[i] < A.n ? A.train.ell[W[i]] : 0.0f);
       // two neighbours per step into two partial sums (independent chains),
       // F = even-rank terms + odd-rank terms
       float F0 = 0.0f, F1 = 0.0f;
@@ -1185,8 +1226,10 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
           const float e = __fmul_rn(wt, rcp_hw(__fadd_rn(D, ek)));
           if (t & 1u) F1 = __fadd_rn(F1, e);
           else F0 = __fadd_rn(F0, e);
+          if (train) ts.add(P, g2, d2, elli, __fsub_rn(lj, lsh), ci);
         }
         M.F[i] = __fadd_rn(F0, F1);
+        if (train) ts.store(A, W[i], r2i);
         continue;
       }
       // two ranks per step in the two lanes of packed FP32 instructions (even ranks
@@ -1221,9 +1264,15 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         float ta, tb;
         upk2(mul2(pk2(ex2_hw(ea), ex2_hw(eb)), pk2(rcp_hw(qa), rcp_hw(qb))), ta, tb);
         FF = add2(FF, pk2(ta, two ? tb : 0.0f));
+        if (train) {
+          auto ell_of = [&](uint32_t j) { return kPacked ? M.wa[j] : (W[j] < A.n ? A.train.ell[W[j]] : 0.0f); };
+          ts.add(P, g2, da, elli, ell_of(ja), ci);
+          if (two) ts.add(P, g2, db, elli, ell_of(jb), ci);
+        }
       }
       upk2(FF, F0, F1);
       M.F[i] = __fadd_rn(F0, F1);
+      if (train) ts.store(A, W[i], r2i);
     }
   }
   __syncthreads();
