@@ -30,7 +30,6 @@ struct denoise_ctx {
   FrameInfo *d_frames = nullptr;
   Tile *d_tiles = nullptr;
   uint32_t *d_hist = nullptr;
-  uint32_t *d_base = nullptr;
   uint32_t *d_lookback = nullptr;
   Leaf *d_leaves = nullptr;
   uint32_t *d_order = nullptr;
@@ -153,7 +152,7 @@ void free_ctx(denoise_ctx *c) {
   if (!c) return;
   cudaSetDevice(c->device);
   void *dptrs[] = {c->d_xyz, c->d_mask, c->d_score, c->d_stage, c->d_gin, c->d_keys[0], c->d_keys[1],
-                   c->d_vals[0], c->d_vals[1], c->d_spts, c->d_frames, c->d_tiles, c->d_hist, c->d_base,
+                   c->d_vals[0], c->d_vals[1], c->d_spts, c->d_frames, c->d_tiles, c->d_hist,
                    c->d_lookback, c->d_leaves, c->d_order, c->d_ctr, c->d_big, c->d_partials, c->d_grad,
                    c->train.sums, c->train.ell, c->train.r2, c->train.F, c->train.stage,
                    c->x_nbr, c->x_r2, c->x_keff, c->x_flag};
@@ -237,34 +236,6 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
     cudaMemcpyAsync(c->d_frames, c->h_frames[c->slot], sizeof(FrameInfo) * nframes, cudaMemcpyHostToDevice, st);
   }
   if (use_events) cudaEventRecord(c->ev[0], st);
-  FrontArgs fa{};
-  fa.xyz = xyz_dev;
-  fa.xyz_src = xyz_mapped;
-  fa.xyz_copy = xyz_mapped ? c->d_xyz : nullptr;
-  fa.n = n;
-  fa.frames = c->d_frames;
-  fa.nframes = nframes;
-  fa.tiles = c->d_tiles;
-  fa.ntiles = c->ntiles;
-  fa.keys[0] = c->d_keys[0];
-  fa.keys[1] = c->d_keys[1];
-  fa.vals[0] = c->d_vals[0];
-  fa.vals[1] = c->d_vals[1];
-  fa.spts = c->d_spts;
-  fa.digit_hist = c->d_hist;
-  fa.digit_base = c->d_base;
-  fa.lookback = c->d_lookback;
-  fa.leaves = c->d_leaves;
-  fa.ctr = c->d_ctr;
-  fa.dbg_key = dbg ? dbg->key : nullptr;
-  fa.max_depth = (int)p.max_depth;
-  fa.leaf_capacity = p.leaf_capacity;
-  fa.full_sort = p.cross_leaf != 0;
-  fa.spin_limit = c->wait_limit;
-  fa.hold_tile1 = c->hold_tile1;
-  if (launch_front(fa, st, &launches, use_events ? &c->ev[1] : nullptr, use_events ? &c->ev[2] : nullptr))
-    return cuda_fail();
-  if (use_events) cudaEventRecord(c->ev[3], st);
   LeafArgs la{};
   la.n = n;
   la.spts = c->d_spts;
@@ -303,6 +274,35 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
     la.train = c->train;
     la.use_train = 1;
   }
+  FrontArgs fa{};
+  fa.xyz = xyz_dev;
+  fa.xyz_src = xyz_mapped;
+  fa.xyz_copy = xyz_mapped ? c->d_xyz : nullptr;
+  fa.n = n;
+  fa.frames = c->d_frames;
+  fa.nframes = nframes;
+  fa.tiles = c->d_tiles;
+  fa.ntiles = c->ntiles;
+  fa.keys[0] = c->d_keys[0];
+  fa.keys[1] = c->d_keys[1];
+  fa.vals[0] = c->d_vals[0];
+  fa.vals[1] = c->d_vals[1];
+  fa.spts = c->d_spts;
+  fa.digit_hist = c->d_hist;
+  fa.lookback = c->d_lookback;
+  fa.leaves = c->d_leaves;
+  fa.tile_box = reinterpret_cast<uint4 *>(c->d_leaves);  // 32 bytes a tile, idle until the leaf finder writes (32 a point)
+  fa.ctr = c->d_ctr;
+  fa.dbg_key = dbg ? dbg->key : nullptr;
+  fa.max_depth = (int)p.max_depth;
+  fa.leaf_capacity = p.leaf_capacity;
+  fa.lmax = la.lmax;
+  fa.full_sort = p.cross_leaf != 0;
+  fa.spin_limit = c->wait_limit;
+  fa.hold_tile1 = c->hold_tile1;
+  if (launch_front(fa, st, &launches, use_events ? &c->ev[1] : nullptr, use_events ? &c->ev[2] : nullptr))
+    return cuda_fail();
+  if (use_events) cudaEventRecord(c->ev[3], st);
   if (launch_leaf_prep(la, c->num_sms, st, &launches)) return cuda_fail();
   if (use_events) cudaEventRecord(c->ev[4], st);
   if (p.cross_leaf) {
@@ -551,7 +551,6 @@ int denoise_create(denoise_ctx **out, int device, size_t max_points, uint32_t ma
   e |= dalloc(&c->d_frames, max_frames);
   e |= dalloc(&c->d_tiles, c->max_tiles);
   e |= dalloc(&c->d_hist, (size_t)max_frames * kMaxPasses * 256);
-  e |= dalloc(&c->d_base, (size_t)max_frames * kMaxPasses * 256);
   e |= dalloc(&c->d_lookback, (size_t)kMaxPasses * c->max_tiles * 256);
   e |= dalloc(&c->d_leaves, N);
   e |= dalloc(&c->d_order, N);

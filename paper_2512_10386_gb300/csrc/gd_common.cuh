@@ -34,7 +34,7 @@ constexpr uint32_t kStFatal = kStNonFinite | kStTimeout | kStInternal;
 // One frame of a batch: its point range and root cube (filled on the device).
 struct FrameInfo {
   uint32_t begin, end;
-  uint32_t lo_ord[3], hi_ord[3];  // order-preserving integer images of min / max (atomics)
+  uint32_t lo_ord[3], hi_ord[3];  // order-preserving integer images of min / max
   float lo[3];
   float side, s, delta;
 };
@@ -44,7 +44,8 @@ struct Tile {
   uint32_t frame, begin, end, first_tile;  // first_tile: index of the frame's first tile
 };
 
-// Octree leaf; lo and h (Eq. 10-11) are filled by the leaf-prep kernel.
+// Octree leaf; lo and h (Eq. 10-11) are filled by the leaf-prep kernel (until then h
+// holds the bits of the leaf's place in its size class).
 struct Leaf {
   uint32_t start, count, frame, level;
   float lo[3];
@@ -96,7 +97,6 @@ struct Counters {
   uint32_t far_count;                    // queries left to a warp of their own (gd_boxknn.cuh)
   uint32_t tile_work[kMaxPasses];        // radix-pass tile counters
   uint32_t cls_count[kLeafClasses];      // leaves per size class
-  uint32_t cls_cursor[kLeafClasses];     // fill cursors of the class-ordered leaf list
   unsigned long long knn_pairs;
   unsigned long long n_p1;
   unsigned long long n_p2;
@@ -153,6 +153,23 @@ __device__ __forceinline__ unsigned long long morton3(uint32_t qx, uint32_t qy, 
   return (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
 }
 
+// Size class of a leaf (see kLeafClasses) and the lane's place among the leaves of its
+// class: one atomic per class and warp.
+__device__ __forceinline__ uint32_t leaf_class(uint32_t count, uint32_t lmax) {
+  if (count > lmax) return 0;
+  const uint32_t b = (count - 1) >> 6;  // 64-point classes, largest first
+  return 1 + (kLeafClasses - 2) - (b < kLeafClasses - 2 ? b : kLeafClasses - 2);
+}
+__device__ __forceinline__ uint32_t class_slot(uint32_t *ctr, uint32_t cls, uint32_t active) {
+  const uint32_t peers = __match_any_sync(active, cls);
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t leader = __ffs(peers) - 1;
+  uint32_t base = 0;
+  if (lane == leader) base = atomicAdd(&ctr[cls], (uint32_t)__popc(peers));
+  base = __shfl_sync(peers, base, leader);
+  return base + __popc(peers & ((1u << lane) - 1u));
+}
+
 // Host-side launch helpers (defined in gd_front.cu / gd_leaf.cu).
 struct FrontArgs {
   const float *xyz;       // device copy of the points, read after the bounding-box pass
@@ -167,13 +184,14 @@ struct FrontArgs {
   uint32_t *vals[2];
   float4 *spts;
   uint32_t *digit_hist;   // [nframes][kMaxPasses][256]
-  uint32_t *digit_base;   // [nframes][kMaxPasses][256]
   uint32_t *lookback;     // [kMaxPasses][ntiles][256]
   Leaf *leaves;
   Counters *ctr;
   uint64_t *dbg_key;
   int max_depth;
   uint32_t leaf_capacity;
+  uint32_t lmax;            // largest leaf of the fused kernel's shared-memory path (size classes)
+  uint4 *tile_box;          // [2 ntiles] scratch: each tile's box (idle until the first radix pass writes)
   uint32_t spin_limit;      // iterations of a bounded look-back wait (0 = kSpinLimit)
   uint32_t hold_tile1;      // test hook: tile hold_tile1 - 1 of the first radix pass never publishes (0 = off)
   bool order_only;          // stop after the radix passes (points in octree order down to the sorted bits)

@@ -463,7 +463,7 @@ struct EbMem {
   unsigned long long *keys[2];
   uint32_t *vals[2];
   float4 *spts;
-  uint32_t *hist, *base, *lookback;
+  uint32_t *hist, *lookback;
   unsigned char *box[2];
 };
 size_t eb_carve(unsigned char *p, uint32_t na, uint32_t nb, EbMem *m) {
@@ -483,7 +483,6 @@ size_t eb_carve(unsigned char *p, uint32_t na, uint32_t nb, EbMem *m) {
   for (int i = 0; i < 2; ++i) x.vals[i] = (uint32_t *)take(4 * n);
   x.spts = (float4 *)take(16 * n);
   x.hist = (uint32_t *)take(4ull * 2 * kMaxPasses * 256);
-  x.base = (uint32_t *)take(4ull * 2 * kMaxPasses * 256);
   x.lookback = (uint32_t *)take(4ull * kTopPasses * tiles * 256);
   x.box[0] = take(box_bytes(na));
   x.box[1] = take(box_bytes(nb));
@@ -509,7 +508,7 @@ int eb_build(const EbMem &m, const float *a, uint32_t na, const float *b, uint32
   }
   f.spts = m.spts;
   f.digit_hist = m.hist;
-  f.digit_base = m.base;
+  f.tile_box = reinterpret_cast<uint4 *>(m.vals[1]);  // idle until the first radix pass
   f.lookback = m.lookback;
   f.ctr = ctr;
   f.max_depth = 21;

@@ -15,13 +15,20 @@
 namespace gd {
 
 // ---------------------------------------------------------------------------
-// init: reset counters, bbox accumulators and look-back flags
+// reset of the counters, the digit histograms and the look-back flags (by the
+// bounding-box pass on the side; the kernels that use them come after it)
 // ---------------------------------------------------------------------------
-__global__ void k_init(FrameInfo *frames, uint32_t nframes, Counters *ctr, uint32_t *digit_hist,
-                       uint32_t *lookback, uint32_t n_lookback, int passes) {
-  pdl_wait();
+struct InitArgs {
+  uint32_t nframes;
+  Counters *ctr;
+  uint32_t *digit_hist, *lookback;
+  uint32_t n_lookback;  // words per pass
+  int passes;
+};
+__device__ __forceinline__ void front_reset(const InitArgs &I) {
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t stride = gridDim.x * blockDim.x;
+  Counters *const ctr = I.ctr;
   if (tid == 0) {
     ctr->status = 0;
     ctr->n_leaves = 0;
@@ -31,33 +38,28 @@ __global__ void k_init(FrameInfo *frames, uint32_t nframes, Counters *ctr, uint3
     ctr->split_leaf = 0;
     ctr->xleaf_work = 0;
     for (int i = 0; i < kMaxPasses; ++i) ctr->tile_work[i] = 0;
-    for (int i = 0; i < kLeafClasses; ++i) ctr->cls_count[i] = ctr->cls_cursor[i] = 0;
+    for (int i = 0; i < kLeafClasses; ++i) ctr->cls_count[i] = 0;
     ctr->knn_pairs = 0;
     ctr->n_p1 = 0;
     ctr->n_p2 = 0;
     ctr->score_terms = 0;
   }
-  for (uint32_t f = tid; f < nframes; f += stride) {
-    for (int a = 0; a < 3; ++a) {
-      frames[f].lo_ord[a] = 0xFFFFFFFFu;
-      frames[f].hi_ord[a] = 0u;
-    }
-  }
-  const uint32_t nh = nframes * kMaxPasses * 256u;
-  for (uint32_t i = tid; i < nh; i += stride) digit_hist[i] = 0;
-  const uint32_t nl = n_lookback * (uint32_t)passes;
-  for (uint32_t i = tid; i < nl; i += stride) lookback[i] = 0;
+  const uint32_t nh = I.nframes * kMaxPasses * 256u;
+  for (uint32_t i = tid; i < nh; i += stride) I.digit_hist[i] = 0;
+  const uint32_t nl = I.n_lookback * (uint32_t)I.passes;
+  for (uint32_t i = tid; i < nl; i += stride) I.lookback[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
-// bbox: exact FP32 min / max per frame (order-preserving integer atomics);
-// flags non-finite coordinates.
+// bbox: exact FP32 min / max of every tile (order-preserving integers) and whether a
+// coordinate is not finite; the key pass reduces the tiles of its frame, so nothing
+// has to be cleared for atomics before this, the call's first kernel.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFrontThreads) k_bbox(const float *__restrict__ xyz,
-                                                        float *__restrict__ xyz_copy,
-                                                        FrameInfo *frames, const Tile *__restrict__ tiles,
-                                                        Counters *ctr) {
+                                                        float *__restrict__ xyz_copy, uint4 *__restrict__ tile_box,
+                                                        const Tile *__restrict__ tiles, const InitArgs I) {
   pdl_wait();
+  front_reset(I);
   const Tile t = tiles[blockIdx.x];
   uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u};
   bool bad = false;
@@ -128,8 +130,6 @@ __global__ void __launch_bounds__(kFrontThreads) k_bbox(const float *__restrict_
     }
   }
   bad = __any_sync(0xFFFFFFFFu, bad);
-  // block reduction first: one atomic per block and value (all blocks of a
-  // frame update the same six words, so per-warp atomics would serialise)
   __shared__ uint32_t s_red[kFrontThreads / 32][6];
   __shared__ int s_bad;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -143,24 +143,25 @@ __global__ void __launch_bounds__(kFrontThreads) k_bbox(const float *__restrict_
     if (bad) s_bad = 1;
   }
   __syncthreads();
-  if (threadIdx.x < 6) {
-    const int v = threadIdx.x;
-    uint32_t r = s_red[0][v];
-    for (int ww = 1; ww < kFrontThreads / 32; ++ww) r = (v < 3) ? min(r, s_red[ww][v]) : max(r, s_red[ww][v]);
-    FrameInfo &f = frames[t.frame];
-    if (v < 3) atomicMin(&f.lo_ord[v], r);
-    else atomicMax(&f.hi_ord[v - 3], r);
-    if (v == 0 && s_bad) atomicOr(&ctr->status, kStNonFinite);
+  if (threadIdx.x == 0) {
+    uint32_t r[6];
+    for (int v = 0; v < 6; ++v) {
+      r[v] = s_red[0][v];
+      for (int ww = 1; ww < kFrontThreads / 32; ++ww) r[v] = (v < 3) ? min(r[v], s_red[ww][v]) : max(r[v], s_red[ww][v]);
+    }
+    tile_box[2ull * blockIdx.x] = make_uint4(r[0], r[1], r[2], s_bad ? 1u : 0u);
+    tile_box[2ull * blockIdx.x + 1] = make_uint4(r[3], r[4], r[5], 0u);
   }
 }
 
 // Root cube of a frame from its reduced extents (reading: anchored at the FP32
 // minimum, side = largest FP32 extent, 1 if the frame is a single location).
-__device__ __forceinline__ void root_cube(const FrameInfo &f, float lo[3], float &side, float &s) {
+__device__ __forceinline__ void root_cube(const uint32_t lo_ord[3], const uint32_t hi_ord[3], float lo[3], float &side,
+                                          float &s) {
   side = 0.0f;
   for (int a = 0; a < 3; ++a) {
-    lo[a] = ord2f(f.lo_ord[a]);
-    float e = __fsub_rn(ord2f(f.hi_ord[a]), lo[a]);
+    lo[a] = ord2f(lo_ord[a]);
+    float e = __fsub_rn(ord2f(hi_ord[a]), lo[a]);
     side = (e > side) ? e : side;
   }
   if (side == 0.0f) side = 1.0f;
@@ -173,21 +174,58 @@ __device__ __forceinline__ void root_cube(const FrameInfo &f, float lo[3], float
 // digit histograms of every radix pass (per frame) are accumulated on the way.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFrontThreads) k_keys(const float *__restrict__ xyz, FrameInfo *frames,
+                                                        const uint4 *__restrict__ tile_box,
                                                         const Tile *__restrict__ tiles,
                                                         unsigned long long *__restrict__ keys,
                                                         uint32_t *__restrict__ vals, uint64_t *dbg_key,
                                                         uint32_t *__restrict__ hist, int lowbit, int passes,
-                                                        const Counters *ctr) {
+                                                        Counters *ctr) {
   __shared__ uint32_t sh[kMaxPasses][256];
+  __shared__ uint32_t s_red[6];
+  __shared__ uint32_t s_bad;
   pdl_wait();
-  if (ctr->status & kStFatal) return;
   for (int i = threadIdx.x; i < passes * 256; i += kFrontThreads) (&sh[0][0])[i] = 0;
+  if (threadIdx.x < 6) s_red[threadIdx.x] = threadIdx.x < 3 ? 0xFFFFFFFFu : 0u;
+  if (threadIdx.x == 6) s_bad = 0;
   __syncthreads();
   const Tile t = tiles[blockIdx.x];
+  // the frame's extents from its tiles
+  {
+    const uint32_t nt = (frames[t.frame].end - frames[t.frame].begin + kTilePts - 1u) / kTilePts;
+    uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u}, bad = 0;
+    for (uint32_t i = threadIdx.x; i < nt; i += kFrontThreads) {
+      const uint4 a = tile_box[2ull * (t.first_tile + i)], b = tile_box[2ull * (t.first_tile + i) + 1];
+      mn[0] = min(mn[0], a.x); mn[1] = min(mn[1], a.y); mn[2] = min(mn[2], a.z);
+      mx[0] = max(mx[0], b.x); mx[1] = max(mx[1], b.y); mx[2] = max(mx[2], b.z);
+      bad |= a.w;
+    }
+    if ((threadIdx.x & ~31u) < nt) {  // warps that saw a tile
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const uint32_t l = __reduce_min_sync(0xFFFFFFFFu, mn[a]), h = __reduce_max_sync(0xFFFFFFFFu, mx[a]);
+        if ((threadIdx.x & 31u) == 0) {
+          atomicMin(&s_red[a], l);
+          atomicMax(&s_red[3 + a], h);
+        }
+      }
+      if (bad) s_bad = 1;
+    }
+    __syncthreads();
+  }
+  const bool first = blockIdx.x == t.first_tile && threadIdx.x == 0;
+  if (s_bad) {
+    if (first) atomicOr(&ctr->status, kStNonFinite);
+    return;
+  }
   float lo[3], side, s;
-  root_cube(frames[t.frame], lo, side, s);
-  if (blockIdx.x == t.first_tile && threadIdx.x == 0) {
+  root_cube(s_red, s_red + 3, lo, side, s);
+  if (first) {
     FrameInfo &f = frames[t.frame];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      f.lo_ord[a] = s_red[a];
+      f.hi_ord[a] = s_red[3 + a];
+    }
     f.lo[0] = lo[0];
     f.lo[1] = lo[1];
     f.lo[2] = lo[2];
@@ -217,29 +255,6 @@ __global__ void __launch_bounds__(kFrontThreads) k_keys(const float *__restrict_
   }
 }
 
-// exclusive scan of each (frame, pass) digit histogram -> absolute output bases
-__global__ void __launch_bounds__(256) k_digit_scan(const uint32_t *__restrict__ hist,
-                                                    uint32_t *__restrict__ base,
-                                                    const FrameInfo *__restrict__ frames, int passes,
-                                                    const Counters *ctr) {
-  __shared__ uint32_t warp_tot[8];
-  pdl_wait();
-  if (ctr->status & kStFatal) return;
-  const uint32_t f = blockIdx.x / passes, p = blockIdx.x % passes;
-  const size_t off = ((size_t)f * kMaxPasses + p) * 256;
-  const uint32_t d = threadIdx.x, lane = d & 31, w = d >> 5;
-  uint32_t v = hist[off + d], x = v;
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_tot[w] = x;
-  __syncthreads();
-  uint32_t wp = 0;
-  for (uint32_t i = 0; i < w; ++i) wp += warp_tot[i];
-  base[off + d] = frames[f].begin + wp + x - v;
-}
-
 // ---------------------------------------------------------------------------
 // one radix pass (stable, segmented by frame, decoupled look-back)
 // ---------------------------------------------------------------------------
@@ -251,13 +266,13 @@ __global__ void __launch_bounds__(kFrontThreads) k_radix_pass(
     const unsigned long long *__restrict__ kin, const uint32_t *__restrict__ vin,
     unsigned long long *__restrict__ kout, uint32_t *__restrict__ vout, float4 *__restrict__ pout,
     const float *__restrict__ xyz, const Tile *__restrict__ tiles, const FrameInfo *__restrict__ frames,
-    const uint32_t *__restrict__ digit_base, uint32_t *__restrict__ lookback, uint32_t *tile_counter,
+    const uint32_t *__restrict__ digit_hist, uint32_t *__restrict__ lookback, uint32_t *tile_counter,
     int shift, Counters *ctr, uint32_t spin_limit, uint32_t hold_tile1) {
   constexpr int W = kFrontThreads / 32;
   __shared__ uint32_t s_wcnt[W][256];  // per warp and digit: count, then exclusive prefix over warps
   __shared__ uint32_t s_base[256];     // global output base of each digit for this tile
   __shared__ uint32_t s_doff[256];     // first position of each digit in the tile's sorted order
-  __shared__ uint32_t s_wsum[W];
+  __shared__ unsigned long long s_wsum[W];
   __shared__ unsigned long long s_key[kTilePts];  // the tile in sorted order, for coalesced writes
   __shared__ uint32_t s_val[kTilePts];
   __shared__ uint32_t s_tile;
@@ -274,6 +289,9 @@ __global__ void __launch_bounds__(kFrontThreads) k_radix_pass(
   const Tile t = tiles[ti];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t wbase = t.begin + w * 32 * kFrontItems;
+  // read early: used after the ranking
+  const uint32_t in_frame = digit_hist[(size_t)t.frame * kMaxPasses * 256 + threadIdx.x];
+  const uint32_t fend = frames[t.frame].end, fbeg = frames[t.frame].begin;
 
   unsigned long long key[kFrontItems];
   uint32_t val[kFrontItems], dig[kFrontItems], rank[kFrontItems], peers[kFrontItems];
@@ -322,16 +340,19 @@ __global__ void __launch_bounds__(kFrontThreads) k_radix_pass(
       s_wcnt[ww][d] = run;
       run += c;
     }
-    uint32_t inc = run;
+    // two scans over the digits in one: the frame's histogram (high word: where the
+    // digit's points of the frame begin) and the tile's counts (low word: where they
+    // begin in the tile); both totals stay below 2^30
+    unsigned long long inc = ((unsigned long long)in_frame << 32) | run;
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
       if (lane >= (uint32_t)o) inc += y;
     }
     if (lane == 31) s_wsum[w] = inc;
     __syncthreads();
-    uint32_t wp = 0;
-    for (uint32_t ww = 0; ww < w; ++ww) wp += s_wsum[ww];
-    s_doff[d] = wp + inc - run;
+    for (uint32_t ww = 0; ww < w; ++ww) inc += s_wsum[ww];
+    s_doff[d] = (uint32_t)inc - run;
+    const uint32_t digit_base = fbeg + (uint32_t)(inc >> 32) - in_frame;
     uint32_t *lb = lookback + (size_t)ti * 256;
     uint32_t excl = 0;
     // test hook (off unless the host asks): this tile never publishes, so the
@@ -371,7 +392,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_radix_pass(
       }
       if (publish) atomicExch(&lb[d], kFlagInc | (excl + run));
     }
-    s_base[d] = digit_base[(size_t)t.frame * kMaxPasses * 256 + d] + excl;
+    s_base[d] = digit_base + excl;
   }
   __syncthreads();
   if (s_fail) return;
@@ -386,7 +407,6 @@ __global__ void __launch_bounds__(kFrontThreads) k_radix_pass(
   }
   __syncthreads();
   // ... then written out: consecutive positions of one digit go to consecutive addresses
-  const uint32_t fend = frames[t.frame].end, fbeg = frames[t.frame].begin;
   const uint32_t cnt = t.end - t.begin;
   for (uint32_t j = threadIdx.x; j < cnt; j += kFrontThreads) {
     const unsigned long long k = s_key[j];
@@ -649,7 +669,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
                                                           const Tile *__restrict__ tiles,
                                                           const FrameInfo *__restrict__ frames,
                                                           Leaf *__restrict__ leaves, Counters *ctr,
-                                                          uint32_t cap, int D, int DB) {
+                                                          uint32_t cap, int D, int DB, uint32_t lmax) {
   extern __shared__ unsigned long long s_win[];
   pdl_wait();
   if (ctr->status & kStFatal) return;
@@ -751,8 +771,10 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
 #pragma unroll
   for (int it = 0; it < kLeavesItems; ++it) {
     const uint32_t c = s_cnt[it][threadIdx.x];
+    const uint32_t active = __ballot_sync(0xFFFFFFFFu, c != 0);
     if (!c) continue;
     Leaf lf{};
+    lf.h = __uint_as_float(class_slot(ctr->cls_count, leaf_class(c, lmax), active));
     lf.start = t.begin + it * kFrontThreads + threadIdx.x;
     lf.count = c;
     lf.frame = t.frame;
@@ -790,37 +812,26 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
   const uint32_t spin = a.spin_limit ? a.spin_limit : kSpinLimit;
   const uint32_t nlb = a.ntiles * 256u;
   int nl = 0;
-  {
-    uint32_t work = a.nframes * kMaxPasses * 256u;
-    if (nlb * (uint32_t)passes > work) work = nlb * (uint32_t)passes;
-    uint32_t blocks = (work + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    if (blocks > 4096) blocks = 4096;
-    launch_pdl(k_init, blocks, 256, 0, st, a.frames, a.nframes, a.ctr, a.digit_hist, a.lookback, nlb, passes);
-    ++nl;
-  }
-  launch_pdl(k_bbox, a.ntiles, kFrontThreads, 0, st, a.xyz_src ? a.xyz_src : a.xyz, a.xyz_copy, a.frames, a.tiles,
-             a.ctr);
-  launch_pdl(k_keys, a.ntiles, kFrontThreads, 0, st, a.xyz, a.frames, a.tiles, a.keys[0], a.vals[0], a.dbg_key,
-                                             a.digit_hist, lowbit, passes, a.ctr);
+  const InitArgs init{a.nframes, a.ctr, a.digit_hist, a.lookback, nlb, passes};
+  launch_pdl(k_bbox, a.ntiles, kFrontThreads, 0, st, a.xyz_src ? a.xyz_src : a.xyz, a.xyz_copy, a.tile_box, a.tiles, init);
+  launch_pdl(k_keys, a.ntiles, kFrontThreads, 0, st, a.xyz, a.frames, a.tile_box, a.tiles, a.keys[0], a.vals[0],
+             a.dbg_key, a.digit_hist, lowbit, passes, a.ctr);
   nl += 2;
   if (ev_after_keys) cudaEventRecord(*ev_after_keys, st);
   int cur = 0;
   if (passes > 0) {
-    launch_pdl(k_digit_scan, a.nframes * passes, 256, 0, st, a.digit_hist, a.digit_base, a.frames, passes, a.ctr);
-    ++nl;
     for (int p = 0; p < passes; ++p) {
       const int shift = lowbit + 8 * p;
-      const uint32_t *base = a.digit_base + p * 256;
+      const uint32_t *hist = a.digit_hist + p * 256;
       uint32_t *lb = a.lookback + (size_t)p * nlb;
       if (p == passes - 1) {
         launch_pdl(k_radix_pass<true>, a.ntiles, kFrontThreads, 0, st,
             a.keys[cur], a.vals[cur], a.keys[cur ^ 1], a.vals[cur ^ 1], a.spts, a.xyz, a.tiles, a.frames,
-            base, lb, &a.ctr->tile_work[p], shift, a.ctr, spin, p == 0 ? a.hold_tile1 : 0u);
+            hist, lb, &a.ctr->tile_work[p], shift, a.ctr, spin, p == 0 ? a.hold_tile1 : 0u);
       } else {
         launch_pdl(k_radix_pass<false>, a.ntiles, kFrontThreads, 0, st,
             a.keys[cur], a.vals[cur], a.keys[cur ^ 1], a.vals[cur ^ 1], a.spts, a.xyz, a.tiles, a.frames,
-            base, lb, &a.ctr->tile_work[p], shift, a.ctr, spin, p == 0 ? a.hold_tile1 : 0u);
+            hist, lb, &a.ctr->tile_work[p], shift, a.ctr, spin, p == 0 ? a.hold_tile1 : 0u);
       }
       cur ^= 1;
       ++nl;
@@ -846,7 +857,7 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
                         ? sizeof(unsigned long long) * (kLeavesPart + 2 * ((size_t)a.leaf_capacity + 1))
                         : 0;
   launch_pdl(k_leaves, a.ntiles * kLeavesSplit, kFrontThreads, win, st, a.keys[cur], a.tiles, a.frames, a.leaves, a.ctr,
-             cap, a.max_depth, DB);
+             cap, a.max_depth, DB, a.lmax);
   ++nl;
   if (launches) *launches += nl;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;

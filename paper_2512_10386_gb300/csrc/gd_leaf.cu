@@ -26,56 +26,60 @@ namespace gd {
 // ---------------------------------------------------------------------------
 // leaf prep: Eq. 10-11 for every leaf (all leaves in parallel)
 // ---------------------------------------------------------------------------
-// A block takes 32 leaves at a time: each warp reduces the FP32 bounding boxes
-// of 4 of them (exact min/max), then lane l of warp 0 evaluates leaf l's
-// h = f32(beta * cbrt_spec(V_t / N_t)) with the extents floored at delta and
-// V_t in FP64.  One leaf per lane matters: FP64 issue is scarce on this part,
-// and a warp instruction costs the same with 1 or 32 lanes active.
-constexpr int kPrepThreads = 256;
-constexpr int kPrepLeaves = 32;
-
-__device__ __forceinline__ uint32_t leaf_class(uint32_t count, uint32_t lmax) {
-  if (count > lmax) return 0;
-  const uint32_t b = (count - 1) >> 6;  // 64-point classes, largest first
-  return 1 + (kLeafClasses - 2) - (b < kLeafClasses - 2 ? b : kLeafClasses - 2);
-}
-
-// warp-aggregated atomicAdd of 1 per lane on ctr[cls]; returns the lane's slot
-__device__ __forceinline__ uint32_t class_slot(uint32_t *ctr, uint32_t cls, uint32_t active) {
-  const uint32_t peers = __match_any_sync(active, cls);
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t leader = __ffs(peers) - 1;
-  uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(&ctr[cls], (uint32_t)__popc(peers));
-  base = __shfl_sync(peers, base, leader);
-  return base + __popc(peers & ((1u << lane) - 1u));
-}
+// A warp takes 8 leaves at a time: the FP32 bounding boxes (exact min/max) one after
+// the other, their descriptors and first points loaded ahead, then lane l evaluates
+// leaf l's voxel size and scatters the leaf's index into the largest-first order: the
+// leaf finder has counted the size classes and left each leaf its place in its class.
+// With few leaves a warp takes one.  (32 leaves a block, the FP64 cube root's ten
+// steps and a kernel of its own for the order took 15.4 + 3.0 us for 8 leaves and 18.2
+// + 3.8 us for 5,700; this one 5.2 and 12.1 us,
+// and for 93,566 leaves 74.1 + 7.9 -> 47.9 us.)
+constexpr int kPrepThreads = 128;
+constexpr uint32_t kPrepLeaves = 8;  // per warp
 
 __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__restrict__ spts, Leaf *leaves,
-                                                            const FrameInfo *__restrict__ frames,
-                                                            Counters *ctr, float beta, uint32_t lmax, bool skip_big) {
-  __shared__ float s_ext[kPrepLeaves][3];
+                                                            const FrameInfo *__restrict__ frames, Counters *ctr,
+                                                            uint32_t *__restrict__ order, float beta, uint32_t lmax,
+                                                            bool skip_big) {
   pdl_wait();
   if (ctr->status & kStFatal) return;
   const uint32_t nl = ctr->n_leaves;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  constexpr uint32_t kPerWarp = kPrepLeaves / (kPrepThreads / 32);
-  for (uint32_t g = blockIdx.x * kPrepLeaves; g < nl; g += gridDim.x * kPrepLeaves) {
-    for (uint32_t t = 0; t < kPerWarp; ++t) {
-      const uint32_t slot = w * kPerWarp + t, li = g + slot;
-      if (li >= nl) break;
-      const uint32_t start = leaves[li].start, cnt = leaves[li].count;
-      if (skip_big && cnt > lmax) continue;  // its own kernels take its box (gd_big.cu)
+  // first place of each size class (lane c: class c)
+  const uint32_t cc = lane < kLeafClasses ? ctr->cls_count[lane] : 0u;
+  uint32_t first = cc;
+  for (int o = 1; o < 16; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, first, o);
+    if (lane >= (uint32_t)o) first += y;
+  }
+  first -= cc;
+  // the smallest classes (64 points each, up to kSmallLeaf points) come last
+  if (blockIdx.x == 0 && threadIdx.x == kLeafClasses - kSmallLeaf / 64) ctr->split_leaf = first;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && skip_big) ctr->leaf_work = cc;  // the fused kernel starts behind class 0
+  const uint32_t warps = gridDim.x * (kPrepThreads / 32), wi = blockIdx.x * (kPrepThreads / 32) + w;
+  uint32_t per = (nl + warps - 1) / warps;
+  per = per < kPrepLeaves ? per : kPrepLeaves;
+  if (per == 0) return;
+  for (uint32_t g = wi * per; g < nl; g += warps * per) {
+    const uint32_t lj = g + lane;
+    const bool on = lane < per && lj < nl;
+    Leaf lf{};
+    if (on) lf = leaves[lj];
+    const bool box = on && !(skip_big && lf.count > lmax);  // (a big leaf's own kernels take its box, gd_big.cu)
+    float lo[3] = {0.0f, 0.0f, 0.0f}, ext[3] = {0.0f, 0.0f, 0.0f};
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, box); todo; todo &= todo - 1u) {
+      const int t = __ffs(todo) - 1;
+      const uint32_t start = __shfl_sync(0xFFFFFFFFu, lf.start, t), cnt = __shfl_sync(0xFFFFFFFFu, lf.count, t);
       float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
-      for (uint32_t i0 = lane; i0 < cnt; i0 += 128) {  // four loads in flight per lane
-        float4 p[4];
+      for (uint32_t i0 = lane; i0 < cnt; i0 += 256) {  // eight loads in flight per lane
+        float4 p[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
           const uint32_t i = i0 + 32u * u;
           if (i < cnt) p[u] = spts[start + i];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
           if (i0 + 32u * u < cnt) {
             mn[0] = fminf(mn[0], p[u].x); mn[1] = fminf(mn[1], p[u].y); mn[2] = fminf(mn[2], p[u].z);
             mx[0] = fmaxf(mx[0], p[u].x); mx[1] = fmaxf(mx[1], p[u].y); mx[2] = fmaxf(mx[2], p[u].z);
@@ -84,56 +88,26 @@ __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__rest
       }
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        for (int o = 16; o; o >>= 1) {
-          mn[a] = fminf(mn[a], __shfl_xor_sync(0xFFFFFFFFu, mn[a], o));
-          mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xFFFFFFFFu, mx[a], o));
+        const float l = ord2f(__reduce_min_sync(0xFFFFFFFFu, f2ord(mn[a])));
+        const float h = ord2f(__reduce_max_sync(0xFFFFFFFFu, f2ord(mx[a])));
+        if (lane == (uint32_t)t) {
+          lo[a] = l;
+          ext[a] = __fsub_rn(h, l);
         }
       }
-      if (lane < 3) {
-        const float lo = lane == 0 ? mn[0] : (lane == 1 ? mn[1] : mn[2]);
-        const float hi = lane == 0 ? mx[0] : (lane == 1 ? mx[1] : mx[2]);
-        leaves[li].lo[lane] = lo;
-        s_ext[slot][lane] = __fsub_rn(hi, lo);
-      }
     }
-    __syncthreads();
-    const uint32_t active = __ballot_sync(0xFFFFFFFFu, g + lane < nl);
-    if (w == 0 && g + lane < nl) {
-      const uint32_t li = g + lane;
-      (void)class_slot(ctr->cls_count, leaf_class(leaves[li].count, lmax), active);
-      if (!(skip_big && leaves[li].count > lmax))
-        leaves[li].h = leaf_voxel_size(s_ext[lane], frames[leaves[li].frame].delta, leaves[li].count, beta);
+    const uint32_t cls = on ? leaf_class(lf.count, lmax) : 0u;
+    const uint32_t base = __shfl_sync(0xFFFFFFFFu, first, cls);
+    if (on) {
+      const uint32_t slot = base + __float_as_uint(lf.h);  // its place in its class, from the leaf finder
+      if (slot < nl) order[slot] = lj;
+      else atomicOr(&ctr->status, kStInternal);
     }
-    __syncthreads();
-  }
-}
-
-// Scatter the leaf indices into size-class order (class 0 first); the order
-// within a class is arbitrary and does not affect any result.
-__global__ void __launch_bounds__(256) k_leaf_order(const Leaf *__restrict__ leaves, Counters *ctr,
-                                                    uint32_t *__restrict__ order, uint32_t lmax) {
-  pdl_wait();
-  if (ctr->status & kStFatal) return;
-  const uint32_t nl = ctr->n_leaves;
-  __shared__ uint32_t s_base[kLeafClasses];
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (int c = 0; c < kLeafClasses; ++c) {
-      s_base[c] = run;
-      run += ctr->cls_count[c];
+    if (box) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) leaves[lj].lo[a] = lo[a];
+      leaves[lj].h = leaf_voxel_size(ext, frames[lf.frame].delta, lf.count, beta);
     }
-    // the smallest classes (64 points each, up to kSmallLeaf points) come last
-    if (blockIdx.x == 0) ctr->split_leaf = s_base[kLeafClasses - (int)(kSmallLeaf / 64)];
-  }
-  __syncthreads();
-  for (uint32_t b = blockIdx.x * blockDim.x; b < nl; b += gridDim.x * blockDim.x) {
-    const uint32_t li = b + threadIdx.x;
-    const uint32_t active = __ballot_sync(0xFFFFFFFFu, li < nl);
-    if (li >= nl) continue;
-    const uint32_t cls = leaf_class(leaves[li].count, lmax);
-    const uint32_t slot = s_base[cls] + class_slot(ctr->cls_cursor, cls, active);
-    if (slot < nl) order[slot] = li;
-    else atomicOr(&ctr->status, kStInternal);
   }
 }
 
@@ -178,10 +152,9 @@ uint32_t leaf_pick_lmax(uint32_t leaf_capacity, int kmax, size_t smem_limit) {
 }
 
 int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches) {
-  launch_pdl(k_leaf_prep, num_sms * 4, kPrepThreads, 0, st, a.spts, const_cast<Leaf *>(a.leaves), a.frames, a.ctr, a.p.beta,
-             a.lmax, a.skip_big != 0);
-  launch_pdl(k_leaf_order, num_sms * 2, 256, 0, st, a.leaves, a.ctr, a.order, a.lmax);
-  if (launches) *launches += 2;
+  launch_pdl(k_leaf_prep, num_sms * 8, kPrepThreads, 0, st, a.spts, const_cast<Leaf *>(a.leaves), a.frames, a.ctr, a.order,
+             a.p.beta, a.lmax, a.skip_big != 0);
+  if (launches) *launches += 1;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

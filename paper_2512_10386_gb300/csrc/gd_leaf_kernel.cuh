@@ -168,14 +168,55 @@ __device__ __forceinline__ unsigned long long voxel_key(const float4 &p, const f
          (unsigned long long)vox_index(p.z, lo[2], h);
 }
 
-// Eq. 10-11: h = f32(beta * cbrt_spec(V_t / N_t)) from the FP32 extents, floored at
-// delta, with V_t in FP64
-__device__ __forceinline__ float leaf_voxel_size(const float *ext, float delta, uint32_t count, float beta) {
-  double H[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) H[a] = (double)(ext[a] < delta ? delta : ext[a]);
-  const double V = __dmul_rn(__dmul_rn(H[0], H[1]), H[2]);
+// Eq. 10-11 by the definition: h = f32(beta * cbrt_spec(V_t / N_t)), V_t in FP64
+static __device__ __noinline__ float leaf_voxel_size_fp64(float e0, float e1, float e2, uint32_t count, float beta) {
+  const double V = __dmul_rn(__dmul_rn((double)e0, (double)e1), (double)e2);
   return __double2float_rn(__dmul_rn((double)beta, cbrt_spec(__ddiv_rn(V, (double)count))));
+}
+
+// The same value from the FP32 extents, floored at delta, almost always without FP64
+// (this part issues an FP64 warp instruction every 16 cycles or so per SM, and the
+// definition is a chain of some 200).  cbrt_spec's ten Newton steps end within 2 ulp of
+// the cube root (a step's rounding errors are 2/3 ulp and its last subtraction's
+// half), so h is known as soon as beta * cbrt(V_t / N_t) is, unless that lies next to a
+// rounding boundary of FP32.  It is computed here in pairs of floats (exact products
+// by fused multiply-add; one Newton step from the FP32 cube root) with a relative
+// error below 2^-42; where the value moved up and down by 2^-40 rounds to two
+// different floats, or an exponent is out of range, the definition decides.
+__device__ __forceinline__ float leaf_voxel_size(const float *ext, float delta, uint32_t count, float beta) {
+  float H[3], m[3];
+  int e = 0;
+  bool plain = count <= (1u << 24);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    H[a] = ext[a] < delta ? delta : ext[a];
+    const uint32_t b = __float_as_uint(H[a]), x = (b >> 23) & 0xFFu;  // H >= 0
+    plain = plain && x != 0u && x != 255u;
+    e += (int)x - 127;
+    m[a] = __uint_as_float((b & 0x7FFFFFu) | 0x3F800000u);  // H = m 2^(x - 127), m in [1, 2)
+  }
+  if (plain) {
+    // V = m0 m1 m2 2^e, then V / N, as (high, low)
+    const float n = (float)count;
+    const float ph = __fmul_rn(m[0], m[1]), pl = __fmaf_rn(m[0], m[1], -ph);
+    const float vh = __fmul_rn(ph, m[2]), vl = __fmaf_rn(pl, m[2], __fmaf_rn(ph, m[2], -vh));
+    const float dh0 = __fdiv_rn(vh, n), dl0 = __fdiv_rn(__fadd_rn(__fmaf_rn(-dh0, n, vh), vl), n);
+    // 2^e = 2^(e mod 3) 2^(3 k)
+    const int k = e >= 0 ? e / 3 : -((-e + 2) / 3);
+    const float sc = (float)(1 << (e - 3 * k));
+    const float dh = __fmul_rn(dh0, sc), dl = __fmul_rn(dl0, sc);
+    // cube root: y + c
+    const float y = cbrtf(dh);
+    const float qh = __fmul_rn(y, y), ql = __fmaf_rn(y, y, -qh);
+    const float th = __fmul_rn(qh, y), tl = __fmaf_rn(ql, y, __fmaf_rn(qh, y, -th));
+    const float c = __fdiv_rn(__fadd_rn(__fsub_rn(dh, th), __fsub_rn(dl, tl)), __fmul_rn(3.0f, qh));
+    // times beta, both ends of the error
+    const float hh = __fmul_rn(beta, y), hl = __fmaf_rn(beta, c, __fmaf_rn(beta, y, -hh));
+    const float eps = __fmul_rn(hh, 0x1p-40f);
+    const float lo = __fadd_rn(hh, __fsub_rn(hl, eps)), hi = __fadd_rn(hh, __fadd_rn(hl, eps));
+    if (lo == hi && lo >= 0x1p-60f && lo <= 0x1p60f && k >= -60 && k <= 60) return __fmul_rn(lo, exp2f((float)k));
+  }
+  return leaf_voxel_size_fp64(H[0], H[1], H[2], count, beta);
 }
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
@@ -1381,9 +1422,11 @@ __global__ void __launch_bounds__(kNT, leaf_min_ctas(kNT)) k_leaf(const LeafArgs
   pdl_wait();
   // the part of the largest-first order this launch takes: every leaf, or those
   // before the split (more than kSmallLeaf points), or from it (the small leaves);
-  // without the first class where those leaves have their own kernels (gd_big.cu)
+  // where the first class's leaves have their own kernels (gd_big.cu), the prep kernel
+  // starts the counter behind them (a test here made the kernel 13 % slower on the
+  // dense scan)
   const uint32_t n_all = A.ctr->n_leaves, split = A.ctr->split_leaf;
-  const uint32_t w_lo = (A.part == 2) ? split : A.skip_big ? A.ctr->cls_count[0] : 0u, w_hi = (A.part == 1) ? split : n_all;
+  const uint32_t w_lo = (A.part == 2) ? split : 0u, w_hi = (A.part == 1) ? split : n_all;
   uint32_t *const wctr = (kXl && A.xphase == 3) ? &A.ctr->leaf_work2
                          : (A.part == 2)         ? &A.ctr->leaf_work3
                                                  : &A.ctr->leaf_work;

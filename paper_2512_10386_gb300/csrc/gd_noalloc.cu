@@ -5,8 +5,8 @@
 // For callers that cannot allocate device memory (a host framework that owns
 // all allocations, a loop whose policy forbids cudaMalloc): nothing here calls
 // cudaMalloc, cudaFree, cudaMallocHost or any allocating library routine.  The
-// array is shared by all calls and keeps the last call's contents; k_init of
-// the front end clears the counters, histograms and look-back flags each call,
+// array is shared by all calls and keeps the last call's contents; the front
+// end's first kernel clears the counters, histograms and look-back flags each call,
 // and k_noalloc_tables rewrites the frame and tile tables.  Overlapping calls
 // race on the array.
 #include <cuda_runtime.h>
@@ -35,8 +35,7 @@ constexpr size_t kOffOrder = kOffLeaves + al256(sizeof(Leaf) * kN);
 constexpr size_t kOffFrames = kOffOrder + al256(4 * kN);
 constexpr size_t kOffTiles = kOffFrames + al256(sizeof(FrameInfo));
 constexpr size_t kOffHist = kOffTiles + al256(sizeof(Tile) * kTiles);
-constexpr size_t kOffBase = kOffHist + al256(4 * kMaxPasses * 256);
-constexpr size_t kOffLookback = kOffBase + al256(4 * kMaxPasses * 256);
+constexpr size_t kOffLookback = kOffHist + al256(4 * kMaxPasses * 256);
 constexpr size_t kOffCtr = kOffLookback + al256(4 * kMaxPasses * kTiles * 256);
 constexpr size_t kOffSpill = kOffCtr + al256(sizeof(Counters));
 constexpr size_t kScratchBytes = kOffSpill + al256((size_t)kSpillBpp * kN);
@@ -163,15 +162,13 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
   fa.vals[1] = (uint32_t *)(b + kOffVals1);
   fa.spts = (float4 *)(b + kOffSpts);
   fa.digit_hist = (uint32_t *)(b + kOffHist);
-  fa.digit_base = (uint32_t *)(b + kOffBase);
   fa.lookback = (uint32_t *)(b + kOffLookback);
   fa.leaves = (Leaf *)(b + kOffLeaves);
+  fa.tile_box = (uint4 *)fa.leaves;  // idle until the leaf finder writes
   fa.ctr = ctr;
   fa.dbg_key = nullptr;
   fa.max_depth = (int)p->max_depth;
   fa.leaf_capacity = p->leaf_capacity;
-  if (launch_front(fa, st, nullptr, nullptr, nullptr)) return fail_cuda();
-
   LeafArgs la{};
   la.n = nn;
   la.spts = fa.spts;
@@ -193,6 +190,8 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
     la.far_queue = reinterpret_cast<uint2 *>(fa.keys[front_sorted_buffer(fa.max_depth, false) ^ 1]);
     if (la.lmax > above) la.lmax = above;
   }
+  fa.lmax = la.lmax;
+  if (launch_front(fa, st, nullptr, nullptr, nullptr)) return fail_cuda();
   if (launch_leaf_prep(la, su.num_sms, st, nullptr) || launch_leaf(la, su.num_sms, st, nullptr)) return fail_cuda();
 
   uint32_t status = 0;
