@@ -284,6 +284,8 @@ int launch_big(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches);
 // the recording instantiation (debug / training outputs), in its own translation unit
 int launch_leaf_rec(const LeafArgs &a, int num_sms, cudaStream_t st);
 int launch_leaf_xl(const LeafArgs &a, int num_sms, cudaStream_t st);
+// leaves of at most kSmallLeaf points, from the split of the order on (gd_leaf_tiny.cu)
+int launch_leaf_tiny(const LeafArgs &a, int num_sms, cudaStream_t st);
 
 // Evaluation metrics (Eq. 29-30) and the baseline of Sec. 2.2 (gd_eval.cu).
 struct EvalArgs {

@@ -180,6 +180,18 @@ static uint32_t leaf_auto_threads(uint32_t n, uint32_t lmax) {
   return 512;
 }
 
+// Whether leaves of at most kSmallLeaf points get a warp each (gd_leaf_tiny.cu).  That
+// kernel needs a fifth of the instructions of the fused one for such a leaf, but its
+// long straight code makes the first leaf of a warp slow (50 us: instruction
+// fetches), and its warps take registers from the CTAs of the larger leaves: it pays
+// where small leaves are many.  us a call, fused / tiny: leaf capacity 64, 40k points 113
+// / 128, 100k 162 / 140, 560k 555 / 322; capacity 128, 100k 134 / 151, 200k 191 / 189, 560k
+// 371 / 345; capacity 256, 300k 226 / 230, 560k 347 / 346, 720k (8 LiDAR frames) 463 / 453,
+// 6.1M (64 frames) 3445 / 3221; capacity 512, 560k 400 / 403, 1.1M 837 / 841.
+static bool leaf_tiny_pays(uint32_t n, uint32_t lmax) {
+  return lmax <= 64 ? n >= 80000u : lmax <= 128 ? n >= 250000u : lmax <= 256 && n >= 600000u;
+}
+
 int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launches, cudaStream_t side, cudaEvent_t fork,
                 cudaEvent_t join) {
   LeafArgs a = args;
@@ -196,7 +208,8 @@ int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launche
       return -1;
     return 0;
   }
-  if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a.n, a.lmax);
+  const bool chosen = a.threads == 0 && a.ctas_per_sm == 0;  // the caller leaves the choice open
+  if (chosen) a.threads = leaf_auto_threads(a.n, a.lmax);
   if (a.xphase != 0) {  // the cross-leaf phases: their own instantiation
     if (launches) ++*launches;
     return launch_leaf_xl(a, num_sms, st);
@@ -204,13 +217,13 @@ int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launche
   auto go = [&](const LeafArgs &x, cudaStream_t s) {
     return (x.use_dbg || x.use_train) ? launch_leaf_rec(x, num_sms, s) : launch_threads<false, false>(x, num_sms, s);
   };
-  // A small leaf's per-leaf steps keep few warps busy; on 64-thread CTAs of a
-  // 64-point shared-memory layout twice as many CTAs share an SM.  The large
-  // leaves keep their 128-thread CTAs; the two launches run side by side, and the
-  // small-leaf CTAs take the SMs the large-leaf CTAs leave (the order of the
-  // leaves and every result are the same as with one launch).
-  const bool split = side && fork && join && (a.threads == 0 || a.threads == 128) && a.lmax > kSmallLeaf &&
-                     a.ctas_per_sm == 0;
+  // Leaves of at most kSmallLeaf points beside the others, one warp each
+  // (gd_leaf_tiny.cu), or, where the recording or a structural variant needs the fused
+  // kernel, on 64-thread CTAs of a 64-point shared-memory layout; the others keep their
+  // CTAs, and the order of the leaves and every result are the same as with one launch.
+  const bool tiny = chosen && leaf_tiny_pays(a.n, a.lmax) && !a.use_dbg && !a.use_train && !a.p.stage_off && !a.p.rescore_p2;
+  const bool split = side && fork && join && a.ctas_per_sm == 0 &&
+                     (a.lmax > kSmallLeaf ? a.threads == 0 || a.threads == 128 : tiny);
   if (!split) {
     if (launches) ++*launches;
     return go(a, st);
@@ -218,11 +231,11 @@ int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launche
   LeafArgs big = a, small = a;
   big.part = 1;
   small.part = 2;
-  small.threads = 64;  // (32-thread CTAs: dense scan +1.7 %, 64 LiDAR frames -1.4 %)
+  small.threads = 64;
   small.lmax = kSmallLeaf;
   if (launches) *launches += 2;
   if (cudaEventRecord(fork, st) != cudaSuccess || cudaStreamWaitEvent(side, fork, 0) != cudaSuccess) return -1;
-  if (go(big, st) || go(small, side)) return -1;
+  if (go(big, st) || (tiny ? launch_leaf_tiny(small, num_sms, side) : go(small, side))) return -1;
   if (cudaEventRecord(join, side) != cudaSuccess || cudaStreamWaitEvent(st, join, 0) != cudaSuccess) return -1;
   return 0;
 }
