@@ -663,8 +663,49 @@ static_assert(kLeavesSmemKeys * 8 + kLeavesItems * kFrontThreads * 5 + 64 <= 48 
 // node shared with position i-1 holds more than leaf_capacity points (so the
 // leaf of i is a proper descendant of the deepest shared node, and begins at i).
 // Every search below stays within cap + 1 positions of i, except the one at the
-// maximum depth D; with cap <= kLeavesSmemCap the block first stages its tile's
-// keys plus that halo on both sides in shared memory and searches there.
+// maximum depth D (over `keys`, the whole frame's).  Returns the leaf's count and
+// level, or 0 if no leaf starts at i.
+__device__ __forceinline__ uint32_t find_leaf(const unsigned long long *kb, uint32_t koff,
+                                              const unsigned long long *keys, uint32_t i, uint32_t fb, uint32_t fe,
+                                              uint32_t cap, int D, int DB, int *level) {
+  const unsigned long long ki = kb[i - koff];
+  const uint32_t wlo = (i - fb > cap + 1) ? i - cap - 1 : fb, whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
+  // does the level-l node that holds i-1 and i have more than cap points?
+  auto big = [&](int l) {
+    if (l == 0) return (fe - fb) > cap;
+    const unsigned long long pre = prefix_of(ki, l);
+    return upper_pre(kb, koff, i, whi, pre, l) - lower_pre(kb, koff, wlo, i, pre, l) > cap;
+  };
+  int L;  // level of the first node that starts at i
+  if (i == fb) {
+    L = 0;
+  } else {
+    const unsigned long long x = kb[i - 1 - koff] ^ ki;
+    const int l = (x == 0) ? 21 : (__clzll((long long)x) - 1) / 3;  // shared levels below the root
+    if (l >= D) return 0;                                            // same max-depth node
+    // below level DB the keys are in octree order only inside level-DB nodes of more
+    // than cap points; a smaller one lies inside one leaf, which cannot start at i
+    if (l > DB && !big(DB)) return 0;
+    if (!big(l)) return 0;
+    L = l + 1;
+  }
+  // descend from the level-L node starting at i to the leaf containing i
+  for (;; ++L) {
+    const unsigned long long pre = prefix_of(ki, L);
+    uint32_t e;
+    if (L < D) {
+      e = upper_pre(kb, koff, i, whi, pre, L);
+      if (e - i > cap) continue;
+    } else {
+      e = upper_pre(keys, 0, i, fe, pre, L);  // a max-depth node may be of any size
+    }
+    *level = L;
+    return e - i;  // >= 1: position i is in its own leaf
+  }
+}
+
+// With cap <= kLeavesSmemCap the block first stages its tile's keys plus a halo of cap
+// + 1 on both sides in shared memory and searches there.
 __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long long *__restrict__ keys,
                                                           const Tile *__restrict__ tiles,
                                                           const FrameInfo *__restrict__ frames,
@@ -700,53 +741,9 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
     const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x;
     s_cnt[it][threadIdx.x] = 0;
     if (i >= t.end) continue;
-    const unsigned long long ki = kb[i - koff];
-    int L;  // level of the first node that starts at i
-    if (i == fb) {
-      L = 0;
-    } else {
-      const unsigned long long x = kb[i - 1 - koff] ^ ki;
-      int l = (x == 0) ? 21 : (__clzll((long long)x) - 1) / 3;  // shared levels below the root
-      if (l >= D) continue;                                      // same max-depth node
-      if (l > DB) {
-        // i-1 and i share a level-DB node; below level DB the keys are in octree
-        // order only inside level-DB nodes of more than cap points.  A smaller one
-        // lies inside one leaf, which cannot start at i.
-        const unsigned long long preB = prefix_of(ki, DB);
-        const uint32_t wlo = (i - fb > cap + 1) ? i - cap - 1 : fb;
-        const uint32_t whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
-        if (upper_pre(kb, koff, i, whi, preB, DB) - lower_pre(kb, koff, wlo, i, preB, DB) <= cap) continue;
-      }
-      // count of the level-l node containing i-1 and i, decided within a window
-      bool big;
-      if (l == 0) {
-        big = (fe - fb) > cap;
-      } else {
-        const unsigned long long pre = prefix_of(ki, l);
-        const uint32_t wlo = (i - fb > cap + 1) ? i - cap - 1 : fb;
-        const uint32_t whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
-        const uint32_t a = lower_pre(kb, koff, wlo, i, pre, l);
-        const uint32_t b = upper_pre(kb, koff, i, whi, pre, l);
-        big = (b - a) > cap;
-      }
-      if (!big) continue;
-      L = l + 1;
-    }
-    // descend from the level-L node starting at i to the leaf containing i
-    for (;; ++L) {
-      const unsigned long long pre = prefix_of(ki, L);
-      uint32_t e;
-      if (L < D) {
-        const uint32_t whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
-        e = upper_pre(kb, koff, i, whi, pre, L);
-        if (e - i > cap) continue;
-      } else {
-        e = upper_pre(keys, 0, i, fe, pre, L);  // a max-depth node may be of any size
-      }
-      s_cnt[it][threadIdx.x] = e - i;  // >= 1: position i is in its own leaf
-      s_lvl[it][threadIdx.x] = (uint8_t)L;
-      break;
-    }
+    int L = 0;
+    s_cnt[it][threadIdx.x] = find_leaf(kb, koff, keys, i, fb, fe, cap, D, DB, &L);
+    s_lvl[it][threadIdx.x] = (uint8_t)L;
   }
   // pass 2: one atomic per block reserves the block's leaf slots
   uint32_t mine = 0;
@@ -784,6 +781,283 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
 }
 
 // ---------------------------------------------------------------------------
+// one small frame: everything above in one block
+// ---------------------------------------------------------------------------
+// A call of a few thousand points spent 60 us in nine kernels of one or two tiles each,
+// every one a launch and a chain of dependent reads.  Up to kSmallFront points one
+// block does it all from shared memory: extents, keys, a bitonic sort of (sorted key
+// bits, input index), the big level-DB nodes' order, leaves and their size classes; the
+// prep kernel follows as ever.  1,500 points, whole call:
+// 120.6 -> 103.6 us.
+constexpr uint32_t kSmallFront = 4096;
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallItems = (int)kSmallFront / kSmallThreads;
+constexpr size_t kSmallSmem = (size_t)kSmallFront * 16;
+
+struct SmallArgs {
+  const float *xyz;
+  float *xyz_copy;
+  uint32_t n;
+  FrameInfo *frame;
+  unsigned long long *keys;  // sorted keys out
+  float4 *spts;
+  Leaf *leaves;
+  Counters *ctr;
+  uint64_t *dbg_key;
+  uint32_t cap, lmax;
+  int D, DB, lowbit, key_low;
+};
+
+// ascending bitonic sort of N = kSmallThreads * E values, thread t holding t*E .. t*E+E-1;
+// partners up to 32*E apart through shuffles, the others through buf
+template <int E>
+__device__ __forceinline__ void small_sort(unsigned long long (&v)[E], unsigned long long *buf, uint32_t N) {
+  const uint32_t t = threadIdx.x;
+#pragma unroll 1
+  for (uint32_t size = 2; size <= N; size <<= 1) {
+#pragma unroll 1
+    for (uint32_t j = size >> 1; j > 0; j >>= 1) {
+      if (j < (uint32_t)E) {
+#pragma unroll
+        for (int jj = 1; jj < E; jj <<= 1) {
+          if ((uint32_t)jj != j) continue;
+#pragma unroll
+          for (int k = 0; k < E; ++k) {
+            const int l = k ^ jj;
+            if (l > k) {
+              const bool asc = ((t * E + k) & size) == 0;
+              const unsigned long long x = v[k], y = v[l];
+              const bool sw = (x > y) == asc;
+              v[k] = sw ? y : x;
+              v[l] = sw ? x : y;
+            }
+          }
+        }
+      } else if (j < 32u * E) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+          const uint32_t e = t * E + k;
+          const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, v[k], j / E);
+          const bool take_min = ((e & j) == 0) == ((e & size) == 0);
+          v[k] = take_min ? (v[k] < y ? v[k] : y) : (v[k] < y ? y : v[k]);
+        }
+      } else {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < E; ++k) buf[t * E + k] = v[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+          const uint32_t e = t * E + k;
+          const unsigned long long y = buf[e ^ j];
+          const bool take_min = ((e & j) == 0) == ((e & size) == 0);
+          v[k] = take_min ? (v[k] < y ? v[k] : y) : (v[k] < y ? y : v[k]);
+        }
+      }
+    }
+  }
+}
+
+// the sort of one call: a composite (sorted key bits, index) per item, padding behind
+template <int E>
+__device__ __forceinline__ void small_order(const unsigned long long *full, unsigned long long *buf, uint32_t n,
+                                            int lowbit) {
+  const uint32_t t = threadIdx.x;
+  unsigned long long v[E];
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const uint32_t i = t * E + k;
+    v[k] = i < n ? ((full[i] >> lowbit) << 32) | i : ~0ull;  // lowbit >= 31: at most 32 key bits
+  }
+  uint32_t N = 2;
+  while (N < n) N <<= 1;
+  small_sort<E>(v, buf, N);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < E; ++k) buf[t * E + k] = v[k];
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_front_small(const SmallArgs A) {
+  extern __shared__ unsigned long long s_dyn[];
+  unsigned long long *const full = s_dyn, *const buf = s_dyn + kSmallFront;  // keys by input index; order
+  __shared__ uint32_t s_red[6], s_bad, s_nl, s_cls[kLeafClasses];
+  __shared__ uint32_t s_wsum[kSmallThreads / 32];
+  pdl_wait();
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5, n = A.n;
+  Counters *const ctr = A.ctr;
+  if (tid < 6) s_red[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
+  if (tid == 6) s_bad = 0;
+  if (tid == 8) s_nl = 0;
+  if (tid < kLeafClasses) s_cls[tid] = 0;
+  __syncthreads();
+  // ---- extents
+  float x[kSmallItems][3];
+  uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u};
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t i = (uint32_t)k * kSmallThreads + tid;
+    if (i < n) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[k][a] = A.xyz[3ull * i + a];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t i = (uint32_t)k * kSmallThreads + tid;
+    if (i < n) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (A.xyz_copy) A.xyz_copy[3ull * i + a] = x[k][a];
+        bad |= !isfinite(x[k][a]);
+        const uint32_t o = f2ord(x[k][a]);
+        mn[a] = min(mn[a], o);
+        mx[a] = max(mx[a], o);
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const uint32_t l = __reduce_min_sync(0xFFFFFFFFu, mn[a]), h = __reduce_max_sync(0xFFFFFFFFu, mx[a]);
+    if (lane == 0) {
+      atomicMin(&s_red[a], l);
+      atomicMax(&s_red[3 + a], h);
+    }
+  }
+  if (bad) s_bad = 1;
+  __syncthreads();
+  if (tid == 0) {  // the call's counters
+    ctr->status = s_bad ? (uint32_t)kStNonFinite : 0u;
+    ctr->leaf_work = ctr->leaf_work2 = ctr->leaf_work3 = ctr->split_leaf = ctr->xleaf_work = 0;
+    ctr->n_leaves = 0;
+    ctr->knn_pairs = ctr->n_p1 = ctr->n_p2 = ctr->score_terms = 0;
+  }
+  if (s_bad) return;
+  float lo[3], side, s;
+  root_cube(s_red, s_red + 3, lo, side, s);
+  if (tid == 0) {
+    FrameInfo &f = *A.frame;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      f.lo_ord[a] = s_red[a];
+      f.hi_ord[a] = s_red[3 + a];
+      f.lo[a] = lo[a];
+    }
+    f.side = side;
+    f.s = s;
+    f.delta = __fmul_rn(side, kInvTwo21);
+  }
+  // ---- keys, order
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t i = (uint32_t)k * kSmallThreads + tid;
+    if (i < n) {
+      const unsigned long long key = morton3(quantise(x[k][0], lo[0], s), quantise(x[k][1], lo[1], s),
+                                             quantise(x[k][2], lo[2], s));
+      full[i] = key;
+      if (A.dbg_key) A.dbg_key[i] = key;
+    }
+  }
+  __syncthreads();
+  if (A.lowbit >= 63) {  // depth 0: the input order
+    for (uint32_t i = tid; i < kSmallFront; i += kSmallThreads) buf[i] = i;
+    __syncthreads();
+  } else if (n <= kSmallThreads) {
+    small_order<1>(full, buf, n, A.lowbit);
+  } else if (n <= 2 * kSmallThreads) {
+    small_order<2>(full, buf, n, A.lowbit);
+  } else {
+    small_order<4>(full, buf, n, A.lowbit);
+  }
+  // ---- the big level-DB nodes in full octree order (rare): one more network over all
+  // items, which outside those nodes compares what it did before
+  if (A.DB < A.D) {
+    const int sh = 63 - 3 * A.DB;
+    auto key_at = [&](uint32_t p) { return full[(uint32_t)buf[p] & 0x7FFFFFFFu]; };  // (the flag set below)
+    bool any = false;
+    for (uint32_t i = tid; i < n; i += kSmallThreads) any |= n - i > A.cap && (key_at(i) >> sh) == (key_at(i + A.cap) >> sh);
+    if (__syncthreads_or(any)) {
+      uint32_t N = 2;
+      while (N < n) N <<= 1;
+      // an item's sort key: everything in a big node, the sorted bits elsewhere
+      auto skey = [&](uint32_t idx, bool big) { return big ? full[idx] >> A.key_low : (full[idx] >> A.lowbit) << (A.lowbit - A.key_low); };
+      for (uint32_t i = tid; i < n; i += kSmallThreads) {
+        const unsigned long long pre = key_at(i) >> sh;
+        uint32_t a = i, b = i + 1;
+        while (a > 0 && i - a <= A.cap && (key_at(a - 1) >> sh) == pre) --a;
+        while (b < n && b - a <= A.cap && (key_at(b) >> sh) == pre) ++b;
+        // the flag travels in the top bit of the index word
+        if (b - a > A.cap) atomicOr(reinterpret_cast<uint32_t *>(buf) + 2 * i, 0x80000000u);
+      }
+      __syncthreads();
+      for (uint32_t size = 2; size <= N; size <<= 1) {
+        for (uint32_t j = size >> 1; j > 0; j >>= 1) {
+          for (uint32_t c = tid; c < (N >> 1); c += kSmallThreads) {
+            const uint32_t a = 2 * j * (c / j) + (c % j), b = a + j;
+            const bool up = (a & size) == 0;
+            const uint32_t ia = (uint32_t)buf[a], ib = (uint32_t)buf[b];
+            // the padding (all ones) sorts last
+            const unsigned long long ka = buf[a] == ~0ull ? ~0ull : skey(ia & 0x7FFFFFFFu, ia >> 31);
+            const unsigned long long kb = buf[b] == ~0ull ? ~0ull : skey(ib & 0x7FFFFFFFu, ib >> 31);
+            const bool less = kb < ka || (kb == ka && (ib & 0x7FFFFFFFu) < (ia & 0x7FFFFFFFu));
+            if (less == up) {
+              const unsigned long long x0 = buf[a];
+              buf[a] = buf[b];
+              buf[b] = x0;
+            }
+          }
+          __syncthreads();
+        }
+      }
+    }
+  }
+  // ---- results in order; then the sorted keys take the order's place.  (Host input is
+  // not read across the link a second time: the device copy was written above.)
+  const float *const src = A.xyz_copy ? A.xyz_copy : A.xyz;
+  unsigned long long sk[kSmallItems];
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t i = (uint32_t)k * kSmallThreads + tid;
+    if (i < n) {
+      const uint32_t v = (uint32_t)buf[i] & 0x7FFFFFFFu;
+      sk[k] = full[v];
+      A.keys[i] = sk[k];
+      A.spts[i] = make_float4(src[3ull * v], src[3ull * v + 1], src[3ull * v + 2], __uint_as_float(v));
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const uint32_t i = (uint32_t)k * kSmallThreads + tid;
+    if (i < n) buf[i] = sk[k];
+  }
+  __syncthreads();
+  // ---- leaves and their size classes
+#pragma unroll 1
+  for (uint32_t i0 = 0; i0 < n; i0 += kSmallThreads) {
+    const uint32_t i = i0 + tid;
+    int L = 0;
+    const uint32_t c = i < n ? find_leaf(buf, 0, buf, i, 0, n, A.cap, A.D, A.DB, &L) : 0u;
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, c != 0);
+    if (lane == 0) s_wsum[w] = m ? atomicAdd(&s_nl, (uint32_t)__popc(m)) : 0u;
+    __syncwarp();
+    if (c) {
+      Leaf lf{};
+      lf.start = i;
+      lf.count = c;
+      lf.level = (uint32_t)L;
+      lf.h = __uint_as_float(atomicAdd(&s_cls[leaf_class(c, A.lmax)], 1u));
+      A.leaves[s_wsum[w] + __popc(m & lanemask_lt())] = lf;
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+  if (tid < kLeafClasses) ctr->cls_count[tid] = s_cls[tid];
+  if (tid == 32) ctr->n_leaves = s_nl;
+}
+
+// ---------------------------------------------------------------------------
 // host launcher
 // ---------------------------------------------------------------------------
 namespace {
@@ -812,6 +1086,18 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
   const uint32_t spin = a.spin_limit ? a.spin_limit : kSpinLimit;
   const uint32_t nlb = a.ntiles * 256u;
   int nl = 0;
+  if (a.nframes == 1 && a.n <= kSmallFront && !a.full_sort && !a.order_only && !a.hold_tile1) {
+    const uint32_t cap = a.leaf_capacity < (1u << 30) ? a.leaf_capacity : (1u << 30);
+    const SmallArgs sa{a.xyz_src ? a.xyz_src : a.xyz, a.xyz_copy, a.n, a.frames, a.keys[passes & 1], a.spts, a.leaves,
+                       a.ctr, a.dbg_key, cap, a.lmax, a.max_depth, DB, passes ? lowbit : 63, key_low};
+    if (cudaFuncSetAttribute(k_front_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem) != cudaSuccess ||
+        launch_pdl(k_front_small, 1, kSmallThreads, kSmallSmem, st, sa) != cudaSuccess)
+      return -1;
+    if (ev_after_keys) cudaEventRecord(*ev_after_keys, st);
+    if (ev_after_sort) cudaEventRecord(*ev_after_sort, st);
+    if (launches) ++*launches;
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  }
   const InitArgs init{a.nframes, a.ctr, a.digit_hist, a.lookback, nlb, passes};
   launch_pdl(k_bbox, a.ntiles, kFrontThreads, 0, st, a.xyz_src ? a.xyz_src : a.xyz, a.xyz_copy, a.tile_box, a.tiles, init);
   launch_pdl(k_keys, a.ntiles, kFrontThreads, 0, st, a.xyz, a.frames, a.tile_box, a.tiles, a.keys[0], a.vals[0],
