@@ -651,13 +651,9 @@ constexpr uint32_t kLeavesSplit = 4;
 constexpr uint32_t kLeavesPart = kTilePts / kLeavesSplit;
 constexpr int kLeavesItems = kFrontItems / kLeavesSplit;
 static_assert(kLeavesPart == (uint32_t)kLeavesItems * kFrontThreads, "whole items per thread");
-// Largest leaf capacity whose key window fits the leaf finder's shared-memory budget
-// (the window and the found-leaf buffer stay within the default 48 KB).
-constexpr uint32_t kLeavesSmemKeys = 5600;  // 43.75 KB of keys
+// Largest leaf capacity whose key window (44 KB) the leaf finder stages in shared memory.
+constexpr uint32_t kLeavesSmemKeys = 5600;
 constexpr uint32_t kLeavesSmemCap = (kLeavesSmemKeys - kLeavesPart) / 2 - 1;
-// static part: found-leaf buffer (kLeavesItems x threads x 5 B) + scan words
-static_assert(kLeavesSmemKeys * 8 + kLeavesItems * kFrontThreads * 5 + 64 <= 48 * 1024,
-              "leaf finder shared memory above the default 48 KB");
 
 // A sorted position i starts a leaf iff it starts its frame, or every octree
 // node shared with position i-1 holds more than leaf_capacity points (so the
@@ -704,8 +700,24 @@ __device__ __forceinline__ uint32_t find_leaf(const unsigned long long *kb, uint
   }
 }
 
-// With cap <= kLeavesSmemCap the block first stages its tile's keys plus a halo of cap
-// + 1 on both sides in shared memory and searches there.
+// shared levels below the root of two keys
+__device__ __forceinline__ int shared_levels(unsigned long long a, unsigned long long b) {
+  const unsigned long long x = a ^ b;
+  return x == 0 ? 21 : (__clzll((long long)x) - 1) / 3;
+}
+
+// With cap <= kLeavesSmemCap the block stages its tile's keys plus a halo of cap + 1 on
+// both sides in shared memory, and the question "does the level-l node of i-1 and i
+// hold more than cap points" is answered for all positions at once.  Such a node
+// exists iff cap + 1 consecutive positions j .. j+cap around i share l levels, that is
+// iff some j in [i-cap, i-1] has shared(j) = shared_levels(key[j], key[j+cap]) >= l: the
+// maximum of shared() over a window of cap positions, built by doubling on bytes, four
+// to a word.  (Keys inside small level-DB nodes are not in octree order, but two keys
+// cap positions apart share level DB only inside a big node, where they are.)  The level
+// of a leaf that starts at i follows from shared(i), and only its count is still
+// searched for.  Two binary searches a position (find_leaf) took 750 warp instructions
+// per 32 points: 64 LiDAR frames 166 -> 96 us, 1.1 M points 41 -> 28 us.
+constexpr uint32_t kLeavesWords = (kLeavesPart + kLeavesSmemCap + 3u) / 4u;
 __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long long *__restrict__ keys,
                                                           const Tile *__restrict__ tiles,
                                                           const FrameInfo *__restrict__ frames,
@@ -721,29 +733,71 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
   t.begin = min(tile.end, tile.begin + part * kLeavesPart);
   t.end = min(tile.end, t.begin + kLeavesPart);
   const uint32_t fb = frames[t.frame].begin, fe = frames[t.frame].end;
-  const unsigned long long *kb = keys;
-  uint32_t koff = 0;
-  if (cap <= kLeavesSmemCap) {  // block-uniform
-    const uint32_t wb = (t.begin - fb > cap + 1) ? t.begin - cap - 1 : fb;
-    const uint32_t we = (fe - t.end > cap + 1) ? t.end + cap + 1 : fe;
-    for (uint32_t i = wb + threadIdx.x; i < we; i += kFrontThreads) s_win[i - wb] = keys[i];
-    __syncthreads();
-    kb = s_win;
-    koff = wb;
-  }
   // pass 1: each thread finds the leaves that start at its items (count, level)
   __shared__ uint32_t s_cnt[kLeavesItems][kFrontThreads];
   __shared__ uint8_t s_lvl[kLeavesItems][kFrontThreads];
   __shared__ uint32_t s_wsum[kFrontThreads / 32];
   __shared__ uint32_t s_base;
+  __shared__ uint32_t s_sh[3][kLeavesWords];  // bytes: shared() + 1 (0: none) from position t.begin - cap on; window maxima
+  if (cap <= kLeavesSmemCap) {  // block-uniform
+    const uint32_t wb = (t.begin - fb > cap + 1) ? t.begin - cap - 1 : fb;
+    const uint32_t we = (fe - t.end > cap + 1) ? t.end + cap + 1 : fe;
+    for (uint32_t i = wb + threadIdx.x; i < we; i += kFrontThreads) s_win[i - wb] = keys[i];
+    __syncthreads();
+    const unsigned long long *const kb = s_win;
+    const uint32_t nw = (cap + (t.end - t.begin) + 3u) / 4u;
+    for (uint32_t q = threadIdx.x; q < nw; q += kFrontThreads) {
+      uint32_t word = 0;
+#pragma unroll
+      for (uint32_t u = 0; u < 4u; ++u) {
+        const uint32_t jc = t.begin + 4u * q + u;  // j + cap
+        if (jc >= fb + cap && jc < fe && jc - t.begin < cap + (t.end - t.begin))
+          word |= (uint32_t)(shared_levels(kb[jc - cap - wb], kb[jc - wb]) + 1) << (8u * u);
+      }
+      s_sh[0][q] = s_sh[1][q] = word;
+    }
+    __syncthreads();
+    uint32_t cur = 1, width = 1;  // s_sh[cur]: maxima over `width` positions
+    for (; 2u * width <= cap; width <<= 1) {
+      for (uint32_t q = threadIdx.x; q < nw; q += kFrontThreads) {
+        const uint32_t v = s_sh[cur][q];
+        auto at = [&](uint32_t x) { return x < nw ? s_sh[cur][x] : 0u; };
+        const uint32_t o = width < 4u ? __funnelshift_r(v, at(q + 1u), 8u * width) : at(q + width / 4u);
+        s_sh[3u - cur][q] = __vmaxu4(v, o);
+      }
+      cur = 3u - cur;
+      __syncthreads();
+    }
+    const uint8_t *const sh = reinterpret_cast<const uint8_t *>(s_sh[0]);
+    const uint8_t *const win = reinterpret_cast<const uint8_t *>(s_sh[cur]);
 #pragma unroll 1
-  for (int it = 0; it < kLeavesItems; ++it) {
-    const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x;
-    s_cnt[it][threadIdx.x] = 0;
-    if (i >= t.end) continue;
-    int L = 0;
-    s_cnt[it][threadIdx.x] = find_leaf(kb, koff, keys, i, fb, fe, cap, D, DB, &L);
-    s_lvl[it][threadIdx.x] = (uint8_t)L;
+    for (int it = 0; it < kLeavesItems; ++it) {
+      const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x, o = i - t.begin;
+      s_cnt[it][threadIdx.x] = 0;
+      if (i >= t.end) continue;
+      const unsigned long long ki = kb[i - wb];
+      int L = 0;
+      if (i != fb) {
+        const int l = shared_levels(kb[i - 1 - wb], ki);
+        if (l >= D || max(win[o], win[o + cap - width]) <= l) continue;
+        L = l + 1;
+      }
+      L = min(D, max(L, (int)sh[o + cap]));
+      const unsigned long long pre = prefix_of(ki, L);
+      const uint32_t whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
+      s_cnt[it][threadIdx.x] = (L < D ? upper_pre(kb, wb, i, whi, pre, L) : upper_pre(keys, 0, i, fe, pre, L)) - i;
+      s_lvl[it][threadIdx.x] = (uint8_t)L;
+    }
+  } else {
+#pragma unroll 1
+    for (int it = 0; it < kLeavesItems; ++it) {
+      const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x;
+      s_cnt[it][threadIdx.x] = 0;
+      if (i >= t.end) continue;
+      int L = 0;
+      s_cnt[it][threadIdx.x] = find_leaf(keys, 0, keys, i, fb, fe, cap, D, DB, &L);
+      s_lvl[it][threadIdx.x] = (uint8_t)L;
+    }
   }
   // pass 2: one atomic per block reserves the block's leaf slots
   uint32_t mine = 0;
@@ -1142,6 +1196,9 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
   const size_t win = (a.leaf_capacity <= kLeavesSmemCap)
                         ? sizeof(unsigned long long) * (kLeavesPart + 2 * ((size_t)a.leaf_capacity + 1))
                         : 0;
+  if (cudaFuncSetAttribute(k_leaves, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kLeavesSmemKeys * sizeof(unsigned long long))) != cudaSuccess)
+    return -1;
   launch_pdl(k_leaves, a.ntiles * kLeavesSplit, kFrontThreads, win, st, a.keys[cur], a.tiles, a.frames, a.leaves, a.ctr,
              cap, a.max_depth, DB, a.lmax);
   ++nl;
