@@ -173,7 +173,7 @@ __device__ __forceinline__ void root_cube(const uint32_t lo_ord[3], const uint32
 // tile of each frame publishes the frame's root cube for later kernels.  The
 // digit histograms of every radix pass (per frame) are accumulated on the way.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kFrontThreads) k_keys(const float *__restrict__ xyz, FrameInfo *frames,
+__global__ void __launch_bounds__(kFrontThreads, 4) k_keys(const float *__restrict__ xyz, FrameInfo *frames,
                                                         const uint4 *__restrict__ tile_box,
                                                         const Tile *__restrict__ tiles,
                                                         unsigned long long *__restrict__ keys,
@@ -189,6 +189,15 @@ __global__ void __launch_bounds__(kFrontThreads) k_keys(const float *__restrict_
   if (threadIdx.x == 6) s_bad = 0;
   __syncthreads();
   const Tile t = tiles[blockIdx.x];
+  float x[kFrontItems][3];  // on their way while the extents are reduced
+#pragma unroll
+  for (int it = 0; it < kFrontItems; ++it) {
+    const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x;
+    if (i < t.end) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[it][a] = xyz[3ull * i + a];
+    }
+  }
   // the frame's extents from its tiles
   {
     const uint32_t nt = (frames[t.frame].end - frames[t.frame].begin + kTilePts - 1u) / kTilePts;
@@ -237,9 +246,9 @@ __global__ void __launch_bounds__(kFrontThreads) k_keys(const float *__restrict_
   for (int it = 0; it < kFrontItems; ++it) {
     const uint32_t i = t.begin + it * kFrontThreads + threadIdx.x;
     if (i < t.end) {
-      const uint32_t q0 = quantise(xyz[3ull * i + 0], lo[0], s);
-      const uint32_t q1 = quantise(xyz[3ull * i + 1], lo[1], s);
-      const uint32_t q2 = quantise(xyz[3ull * i + 2], lo[2], s);
+      const uint32_t q0 = quantise(x[it][0], lo[0], s);
+      const uint32_t q1 = quantise(x[it][1], lo[1], s);
+      const uint32_t q2 = quantise(x[it][2], lo[2], s);
       const unsigned long long k = morton3(q0, q1, q2);
       keys[i] = k;
       vals[i] = i;
