@@ -52,6 +52,12 @@ struct Leaf {
   float h;
 };
 
+// Leaf::level: the octree level in bits 0-4; once the prep kernel has h, and where the
+// leaf's voxel grid (Eq. 12) has at most 2 count cells, bit 31 and the grid's extents in
+// y and z in bits 5-14 and 15-24, for counters addressed by the cell itself.
+constexpr uint32_t kLeafGrid = 1u << 31;
+__host__ __device__ __forceinline__ uint32_t leaf_level(const Leaf &lf) { return lf.level & 31u; }
+
 // The fused leaf kernel takes leaves largest first (longest-processing-time
 // order, so that no large leaf starts last and stretches the tail): class 0 =
 // leaves above the shared-memory size (global-memory path), then classes of 64

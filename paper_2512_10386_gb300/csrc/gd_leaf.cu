@@ -106,7 +106,14 @@ __global__ void __launch_bounds__(kPrepThreads) k_leaf_prep(const float4 *__rest
     if (box) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) leaves[lj].lo[a] = lo[a];
-      leaves[lj].h = leaf_voxel_size(ext, frames[lf.frame].delta, lf.count, beta);
+      const float h = leaf_voxel_size(ext, frames[lf.frame].delta, lf.count, beta);
+      leaves[lj].h = h;
+      // cells a side: the index of the farthest point (vox_index is monotonic), plus one
+      uint32_t g[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) g[a] = vox_index(ext[a], 0.0f, h) + 1u;
+      if (g[0] < 1024u && g[1] < 1024u && g[2] < 1024u && g[0] * g[1] * g[2] <= 2u * lf.count)
+        leaves[lj].level = (lf.level & 31u) | (g[1] << 5) | (g[2] << 15) | kLeafGrid;
     }
   }
 }

@@ -628,17 +628,36 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
   // structural variants (Sec. 4.3.2): stages switched off (A1 voxel gate, A2
   // density gate, A3 score selection) and the score on a kNN within P_2
   const bool a1_on = !(P.stage_off & 1u), a2_on = !(P.stage_off & 2u), a3_on = !(P.stage_off & 4u);
-  // ---- Eq. 12: voxel occupancy (hash with warp-aggregated atomics)
+  // ---- Eq. 12: voxel occupancy, warp-aggregated: one counter per cell of the leaf's
+  // voxel grid where the grid is small (nearly always: V_t / h^3 = N_t / beta^3), else a
+  // hash table of the occupied ones
   const uint32_t hcap = pow2ceil(2 * nt);  // <= the carved capacity
-  for (uint32_t i = tid; i < hcap && a1_on; i += NT) {
-    M.hkey[i] = kEmpty;
+  const bool grid = (lf.level & kLeafGrid) != 0u;
+  const uint32_t gy = (lf.level >> 5) & 1023u, gz = (lf.level >> 15) & 1023u;
+  for (uint32_t i = tid; i < (grid ? 2 * nt : hcap) && a1_on; i += NT) {
+    if (!grid) M.hkey[i] = kEmpty;
     M.hcnt[i] = 0;
   }
   __syncthreads();
   const float lo[3] = {S.lo[0], S.lo[1], S.lo[2]}, h = S.h;
   // each point's hash slot, for the gate below (wa is idle until the score weights)
   uint32_t *const vslot = reinterpret_cast<uint32_t *>(M.wa);
-  for (uint32_t base = 0; base < nt && a1_on; base += NT) {
+  for (uint32_t base = 0; base < nt && a1_on && grid; base += NT) {
+    const uint32_t i = base + tid;
+    uint32_t cell = 0xFFFFFFFFu;
+    if (i < nt) {
+      const float4 p = pts[i];
+      cell = (vox_index(p.x, lo[0], h) * gy + vox_index(p.y, lo[1], h)) * gz + vox_index(p.z, lo[2], h);
+      if (cell >= 2 * nt) {  // cannot happen: the prep kernel measured the grid
+        atomicOr(&A.ctr->status, kStInternal);
+        cell = 0;
+      }
+      vslot[i] = cell;
+    }
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, cell);
+    if (i < nt && (peers & lt) == 0) atomicAdd(M.hcnt + cell, (uint32_t)__popc(peers));
+  }
+  for (uint32_t base = 0; base < nt && a1_on && !grid; base += NT) {
     const uint32_t i = base + tid;
     unsigned long long key = kInvalid;
     if (i < nt) {

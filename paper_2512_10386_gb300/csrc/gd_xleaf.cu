@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kXThreads) k_xleaf_knn(const XleafArgs A) {
     // the 27 cell ranges (level-0 leaf: the whole frame)
     if (tid < 27) {
       uint32_t a = 0, b = 0;
-      const uint32_t L = lf.level;
+      const uint32_t L = leaf_level(lf);
       if (L == 0) {
         if (tid == 13) { a = fr.begin; b = fr.end; }
       } else {
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(128) k_xleaf_ranges(const XleafArgs A) {
     const Leaf lf = A.leaves[li];
     const FrameInfo &fr = A.frames[lf.frame];
     uint32_t a = 0, b = 0;
-    const uint32_t L = lf.level;
+    const uint32_t L = leaf_level(lf);
     if (L == 0) {
       if (lane == 13) {  // a level-0 leaf: the whole frame
         a = fr.begin;
