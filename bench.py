@@ -387,7 +387,7 @@ def run_ours(args):
     achieved = stats["knn_pairs"] * FLOP_PER_PAIR / (leaf_avg_ms / 1000.0) / 1e12
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak_tflops, "traffic": _profile_traffic(),
-                "kernel": "gd::k_leaf<32> (voxel gate + kNN + density gate + score + selection; leaves of more "
+                "kernel": "gd::k_leaf<128> (voxel gate + kNN + density gate + score + selection; leaves of more "
                           "and of at most 64 points in two concurrent launches, timed together)",
                 "work": f"{stats['knn_pairs']} candidate pairs x {FLOP_PER_PAIR:g} FP32 flop per launch",
                 "peak_basis": f"{props.multi_processor_count} SMs x 128 FP32 lanes x 2 flop x {sm_mhz:g} MHz "
@@ -512,11 +512,11 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
       A1/A2/A3     one gate or the score selection switched off (Table 9), on the timed cloud
       rescore_p2   the score on a kNN recomputed within P_2, on the timed cloud
       octree_off   one leaf for the whole cloud (Table 8), on the 36,750-point object cloud
-                   (K = 16): the leaf is one CTA's work, so one SM of the GPU runs it
+                   (K = 16)
       metrics      PSNR / Chamfer distance (Eq. 29-30) between the timed cloud's clean points
-                   and its denoised result (brute-force nearest neighbours both ways)
+                   and its denoised result (nearest neighbours both ways)
       baseline     the gravitational-function method of Sec. 2.2 on the timed cloud
-                   (neighbour counts within R by brute force)"""
+                   (neighbour counts within R)"""
     import torch
 
     import synth
@@ -535,9 +535,12 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
             ms.append(a.elapsed_time(b))
         return float(np.median(ms))
 
-    def entry(points, ms, pairs):
-        return {"points": int(points), "ms": ms, "points_per_s": points / (ms / 1000.0), "pairs": int(pairs),
-                "fp32_frac": pairs * FLOP_PER_PAIR / (ms / 1000.0) / 1e12 / fp32_peak_tflops}
+    def entry(points, ms, pairs, pruned=False):
+        # pruned calls decide over all pairs but compare few of them: no FP32 fraction
+        e = {"points": int(points), "ms": ms, "points_per_s": points / (ms / 1000.0), "pairs": int(pairs)}
+        if not pruned:
+            e["fp32_frac"] = pairs * FLOP_PER_PAIR / (ms / 1000.0) / 1e12 / fp32_peak_tflops
+        return e
 
     n = len(xyz_np)
     xyz = torch.from_numpy(xyz_np).cuda()
@@ -558,7 +561,7 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
         Px = Params(k=32, leaf_capacity=512, cross_leaf=1)
         r = d.run(xyz, Px, stream=stream)
         ms = timed(lambda: d.run(xyz, Px, mask=r.mask, score=r.score, stage=r.stage, stream=stream), 5)
-        out["cross_leaf"] = entry(n, ms, d.stats()["knn_pairs"])
+        out["cross_leaf"] = entry(n, ms, d.stats()["knn_pairs"], pruned=True)
         out["cross_leaf"]["mask_differs_from_leaf_local"] = float((r.mask != ref).float().mean().item())
         d.set_cross_leaf(False)
         clean = torch.from_numpy(np.ascontiguousarray(xyz_np[labels_np == 0])).cuda()
@@ -568,7 +571,7 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
         def metrics():
             m.update(d.eval_metrics(clean, den, stream=stream))
         ms = timed(metrics, 3)
-        out["metrics"] = entry(len(clean) + len(den), ms, 2 * len(clean) * len(den))
+        out["metrics"] = entry(len(clean) + len(den), ms, 2 * len(clean) * len(den), pruned=True)
         out["metrics"].update(clean_points=len(clean), denoised_points=len(den), psnr=m["psnr"],
                               chamfer=m["chamfer"], mse=m["mse"])
         kept = {}
@@ -576,7 +579,7 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
         def baseline():
             kept["n"] = d.run_baseline(xyz, stream=stream)["keep"]
         ms = timed(baseline, 3)
-        out["baseline"] = entry(n, ms, n * n)
+        out["baseline"] = entry(n, ms, n * n, pruned=True)
         out["baseline"]["kept"] = int(kept["n"].sum().item())
     finally:
         d.close()
@@ -587,7 +590,7 @@ def run_variants(xyz_np, labels_np, mask_np, fp32_peak_tflops, stream):
         Po = Params(k=16, leaf_capacity=0xFFFFFFFF)
         r = d.run(xo, Po, stream=stream)
         ms = timed(lambda: d.run(xo, Po, mask=r.mask, score=r.score, stage=r.stage, stream=stream), 2)
-        out["octree_off"] = entry(len(obj), ms, d.stats()["knn_pairs"])
+        out["octree_off"] = entry(len(obj), ms, d.stats()["knn_pairs"], pruned=True)
     finally:
         d.close()
     return out
