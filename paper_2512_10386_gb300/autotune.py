@@ -10,7 +10,7 @@ It measures a workload under candidate settings and keeps the fastest:
   * leaf_smem_points -- largest leaf kept in shared memory; larger leaves take
     the kernel's global-memory path, and each CTA needs less shared memory, so
     more CTAs fit per SM (execution only).
-  * leaf_threads -- 128 (0) or 64 threads per leaf CTA; 64 leaves fewer warps
+  * leaf_threads -- threads per leaf CTA: 0 (by leaf size and cloud) or 64; 64 leaves fewer warps
     idle on small leaves (execution only).  With 64 the CTA count per SM is
     left at the occupancy limit.
 The kNN tile is the whole leaf (it is staged in shared memory at once), so
