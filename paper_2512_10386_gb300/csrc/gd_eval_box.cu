@@ -13,7 +13,7 @@
 //
 // 500,000 against 510,000 points (two passes): 96.8 ms -> 0.95 ms, 0.77 ms of it the
 // four search kernels; counts within 8 % of the extent among 560,000 points: 73.0 ms
-// -> 2.6 ms.  The full pass is bound by the FP32 pipe; these by instruction issue of
+// -> 2.27 ms.  The full pass is bound by the FP32 pipe; these by instruction issue of
 // the box tests and of the chunks that the spheres' borders cross.
 #include "gd_boxes.cuh"
 #include "gd_f32x2.cuh"
@@ -30,8 +30,11 @@ constexpr int kEbThreads = 32 * kEbWarps;
 // Measured, us a call at shares 1 / 2 / 4: object of 30,000 points 266 / 308 / 334,
 // scans of 250,000 709 / 609 / 608 and 500,000 1499 / 1075 / 946.
 inline float nn_share(uint32_t chunks) { return chunks < 2500u ? 1.0f : chunks < 8000u ? 2.0f : 4.0f; }
-constexpr uint32_t kCntList = 1024;  // chunks of the radius count's list
-// A chunk on the list costs its 32 queries together about 190 instructions; a query of
+constexpr uint32_t kCntList = 768;   // chunks of the radius count's list
+constexpr uint32_t kCntBlock = 64;   // of them split into quarters at a time
+constexpr uint32_t kQuarter = kBoxChunk / 4;
+// A chunk on the list costs its 32 queries together about 190 instructions at most (its
+// quarters beyond or within every sphere are dropped first); a query of
 // its own about 600 and 15 for every chunk that straddles its own sphere.  The chunk
 // of queries is left to single-query warps when that is less (queries far apart: the
 // list holds the borders of many spheres).
@@ -44,6 +47,7 @@ struct Cloud {                  // one cloud in octree order
   const float4 *pts;            // x, y, z, index bits in the concatenated input
   uint32_t n, first;            // points, index of the cloud's first point in the concatenation
   BoxIndex box;
+  float4 *quarter;              // boxes of every kQuarter points (radius counts only, else null)
   const unsigned long long *keys;
   const FrameInfo *frame;
 };
@@ -90,6 +94,18 @@ __global__ void __launch_bounds__(kBoxSuper) k_evb_boxes(const Cloud A, const Cl
   if (i < c.n) {
     const float4 p = c.pts[i];
     b = box_point(p.x, p.y, p.z);
+  }
+  if (c.quarter) {
+    Box h = b;
+#pragma unroll
+    for (int o = 1; o < (int)kQuarter; o *= 2) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        h.lo[d] = fminf(h.lo[d], __shfl_xor_sync(0xFFFFFFFFu, h.lo[d], o));
+        h.hi[d] = fmaxf(h.hi[d], __shfl_xor_sync(0xFFFFFFFFu, h.hi[d], o));
+      }
+    }
+    if (i % kQuarter == 0 && i < c.n) box_store(c.quarter, i / kQuarter, h);
   }
   b = box_warp_union(b);
   if (lane == 0) {
@@ -302,29 +318,69 @@ __device__ __forceinline__ uint32_t eb_points(uint32_t first, uint32_t span, uin
   return first < n ? min(span, n - first) : 0u;
 }
 
-// candidates of the listed chunks that lie outside the query's radius
-__device__ __forceinline__ uint32_t eb_beyond(const Cloud &C, EbChunk &S, const uint32_t *list, uint32_t nl, f32x2 QX,
-                                              f32x2 QY, f32x2 QZ, f32x2 R2) {
-  __syncwarp();  // the list is written
+// Compared chunks, not box tests, are most of the count's time, and the shell of
+// chunks that a warp's spheres cut is as thick as the queries' box and the chunk
+// together: boxes of 8 points make the second half as thick on a surface.  us a call
+// before / after (32-point chunks compared whole, their list built twice): 560,000 points of a
+// scan in millimetres 2,635 / 2,270, the same in units of 6.7 mm 667 / 525, object of
+// 560,000 446 / 365, 36,750 283 / 272.  An integer comparison in place of the packed
+// subtraction changed nothing (2,277).
+//
+// The listed chunks: their quarters that lie within the radius of all of the warp's
+// queries go to `whole`, those beyond it of all are dropped, and the others are
+// compared, four at a time (`done` counts such fours); returns the candidates compared
+// that lie outside the lane's radius.
+__device__ __forceinline__ uint32_t eb_border(const Cloud &C, EbChunk &S, const uint32_t *list, uint32_t nl,
+                                              uint32_t *part, const Box &qb, float r2, f32x2 QX, f32x2 QY, f32x2 QZ,
+                                              f32x2 R2, uint32_t &whole, uint32_t &done) {
+  const uint32_t lane = threadIdx.x & 31u;
+  auto fetch = [&](uint32_t four) {
+    const uint32_t p = part[4u * four + lane / kQuarter] * kQuarter + lane % kQuarter;
+    return p < C.n ? C.pts[p] : make_float4(kInf, kInf, kInf, 0.0f);
+  };
   uint32_t beyond = 0;
-  float4 v = nl ? eb_fetch(C, list[0]) : make_float4(0.f, 0.f, 0.f, 0.f);
-  for (uint32_t i = 0; i < nl; ++i) {
-    eb_stage(S, v);
-    if (i + 1 < nl) v = eb_fetch(C, list[i + 1]);  // on its way while this chunk is compared
-    uint32_t bits = 0;  // one bit a candidate, all 32 shifted through
-#pragma unroll
-    for (uint32_t j = 0; j < kBoxChunk; j += 4u) {
-      f32x2 s0, s1;
-      eb_d2x4(S, j, QX, QY, QZ, s0, s1);
-      float e[4];  // the sign of r2 - d^2 is set exactly when d^2 > r2
-      upk2(sub2(R2, s0), e[0], e[1]);
-      upk2(sub2(R2, s1), e[2], e[3]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) bits = __funnelshift_l(__float_as_uint(e[u]), bits, 1);
+  __syncwarp();  // the list is written
+  for (uint32_t base = 0; base < nl; base += kCntBlock) {
+    const uint32_t top = min(nl - base, kCntBlock);
+    uint32_t np = 0;
+    for (uint32_t i = 0; i < top; i += 8u) {
+      const uint32_t e = i + lane / 4u;
+      const uint32_t id = e < top ? list[base + e] * 4u + lane % 4u : 0u;
+      bool edge = false;
+      if (e < top && id * kQuarter < C.n) {
+        const Box b = box_load(C.quarter, id);
+        if (box_upper(b, qb) <= r2)
+          whole += eb_points(id * kQuarter, kQuarter, C.n);
+        else
+          edge = box_lower(b, qb) <= r2;
+      }
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, edge);
+      if (edge) part[np + __popc(m & lanemask_lt())] = id;
+      np += __popc(m);
     }
-    beyond += __popc(bits);
+    if (lane < 3u) part[np + lane] = (C.n + kQuarter - 1u) / kQuarter;  // past the end: at infinite distance
+    __syncwarp();
+    const uint32_t fours = (np + 3u) / 4u;
+    float4 v = fours ? fetch(0) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t i = 0; i < fours; ++i) {
+      eb_stage(S, v);
+      if (i + 1 < fours) v = fetch(i + 1);  // on its way while these are compared
+      uint32_t bits = 0;  // one bit a candidate, all 32 shifted through
+#pragma unroll
+      for (uint32_t j = 0; j < kBoxChunk; j += 4u) {
+        f32x2 s0, s1;
+        eb_d2x4(S, j, QX, QY, QZ, s0, s1);
+        float e[4];  // the sign of r2 - d^2 is set exactly when d^2 > r2
+        upk2(sub2(R2, s0), e[0], e[1]);
+        upk2(sub2(R2, s1), e[2], e[3]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) bits = __funnelshift_l(__float_as_uint(e[u]), bits, 1);
+      }
+      beyond += __popc(bits);
+    }
+    done += fours;
+    __syncwarp();  // the quarters' and the chunks' lists may be written again
   }
-  __syncwarp();  // the list may be written again
   return beyond;
 }
 
@@ -332,10 +388,10 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
                                                           uint32_t *__restrict__ out, uint32_t *__restrict__ far,
                                                           EbWork *work, const Counters *ctr) {
   __shared__ __align__(16) EbChunk s_c[kEbWarps];
-  __shared__ uint32_t s_list[kEbWarps][kCntList];
+  __shared__ uint32_t s_list[kEbWarps][kCntList], s_part[kEbWarps][4u * kCntBlock + 3u];
   if (ctr->status & kStFatal) return;
   EbChunk &S = s_c[threadIdx.x >> 5];
-  uint32_t *const list = s_list[threadIdx.x >> 5];
+  uint32_t *const list = s_list[threadIdx.x >> 5], *const part = s_part[threadIdx.x >> 5];
   const uint32_t lane = threadIdx.x & 31u, nsu = box_supers(C.n), nch = box_chunks(C.n);
   const uint32_t qc = blockIdx.x * kEbWarps + (threadIdx.x >> 5);
   if (qc >= nch) return;
@@ -347,9 +403,9 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
                             __shfl_sync(0xFFFFFFFFu, me.z, 16));
   const f32x2 QX = pk2(me.x, me.x), QY = pk2(me.y, me.y), QZ = pk2(me.z, me.z), R2 = pk2(r2, r2);
   // Boxes within the radius of all of the warp's queries count whole, boxes beyond it
-  // of all count nothing; the chunks between are compared.  The first round only
-  // counts those, for all queries and for one of them, to see whether the queries
-  // belong together.
+  // of all count nothing; the chunks between go on the list.  The first round also
+  // counts those that one of the queries needs, to see whether the queries belong
+  // together; a second one runs where they do and the list was too short for all.
   uint32_t whole = 0, beyond = 0, done = 0, nl = 0, own = 0;
 #pragma unroll 1
   for (int round = 0; round < 2; ++round) {
@@ -361,7 +417,7 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
         in = box_upper(sb, qb) <= r2;
         edge = !in && box_lower(sb, qb) <= r2;
       }
-      if (in && round) whole += eb_points(s * kBoxSuper, kBoxSuper, C.n);
+      if (in) whole += eb_points(s * kBoxSuper, kBoxSuper, C.n);
       uint32_t m = __ballot_sync(0xFFFFFFFFu, edge);
       while (m) {
         const uint32_t c = (s0 + (uint32_t)__ffs(m) - 1u) * 32u + lane;
@@ -374,18 +430,15 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
           ce1 = box_upper(cb, one) > r2 && box_lower(cb, one) <= r2;
         }
         const uint32_t e = __ballot_sync(0xFFFFFFFFu, ce);
-        if (round == 0) {
-          nl += __popc(e);
-          own += __popc(__ballot_sync(0xFFFFFFFFu, ce1));
-          continue;
-        }
         if (ci) whole += eb_points(c * kBoxChunk, kBoxChunk, C.n);
-        if (nl + 32u > kCntList) {  // room for any ballot
-          beyond += eb_beyond(C, S, list, nl, QX, QY, QZ, R2);
-          done += nl;
+        if (round == 0) {
+          own += __popc(__ballot_sync(0xFFFFFFFFu, ce1));
+        } else if (nl + 32u > kCntList) {  // room for any ballot
+          beyond += eb_border(C, S, list, nl, part, qb, r2, QX, QY, QZ, R2, whole, done);
           nl = 0;
         }
-        if (ce) list[nl + __popc(e & lanemask_lt())] = c;
+        const uint32_t at = nl + __popc(e & lanemask_lt());
+        if (ce && at < kCntList) list[at] = c;
         nl += __popc(e);
       }
     }
@@ -394,11 +447,12 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
         if (lane == 0) far[atomicAdd(&work->cnt_far, 1u)] = qc;
         return;
       }
+      if (nl <= kCntList) break;
       nl = 0;
+      whole = 0;
     }
   }
-  beyond += eb_beyond(C, S, list, nl, QX, QY, QZ, R2);
-  done += nl;
+  beyond += eb_border(C, S, list, nl, part, qb, r2, QX, QY, QZ, R2, whole, done);
   whole = __reduce_add_sync(0xFFFFFFFFu, whole);
   if (q < C.n) out[__float_as_uint(me.w) - C.first] = whole + done * kBoxChunk - beyond;
 }
@@ -516,8 +570,10 @@ int eb_build(const EbMem &m, const float *a, uint32_t na, const float *b, uint32
   f.order_only = true;
   if (launch_front(f, st, nullptr, nullptr, nullptr)) return -1;
   const unsigned long long *keys = m.keys[front_sorted_buffer(21, false)];
-  out[0] = Cloud{m.spts, na, 0u, box_index(m.box[0], na), keys, m.frames};
-  out[1] = Cloud{m.spts + na, nb, na, box_index(m.box[1], nb), keys + na, m.frames + 1};
+  // One cloud leaves the concatenation's place free: 16 bytes of quarter boxes for the
+  // 48 of four points (the calls taken here have at least 2^15).
+  out[0] = Cloud{m.spts, na, 0u, box_index(m.box[0], na), nb ? nullptr : reinterpret_cast<float4 *>(m.xyz), keys, m.frames};
+  out[1] = Cloud{m.spts + na, nb, na, box_index(m.box[1], nb), nullptr, keys + na, m.frames + 1};
   k_evb_boxes<<<box_supers(na) + box_supers(nb), kBoxSuper, 0, st>>>(out[0], out[1], ctr);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
