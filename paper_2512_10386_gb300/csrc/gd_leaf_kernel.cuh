@@ -556,8 +556,13 @@ struct PairSum {
   }
   __device__ __forceinline__ double value() const { return __dadd_rn((double)hi, (double)lo); }
 };
+// t ln(d^2) D / (D + eps_k) by the definition
+static __device__ __noinline__ double gamma_term(float t, float l, float D, float ek) {
+  return __dmul_rn(__dmul_rn((double)t, (double)l), __ddiv_rn((double)D, __dadd_rn((double)D, (double)ek)));
+}
 struct TrainSums {
   PairSum w, d, g;
+  double gx = 0.0;
   __device__ __forceinline__ void add(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
     const float lw2 = __fadd_rn(elli, ellj);  // log2 W_ij
     const float D = g2 ? d2 : exp2f(0.5f * P.gamma * log2f(d2));
@@ -566,10 +571,16 @@ struct TrainSums {
     if (t == 0.0f) return;  // (a neighbour of density 0 has ln W = -infinity)
     w.add(t, __fmul_rn(lw2, 0.6931471805599453f));  // ln W_ij
     d.add(t, d2);
-    if (d2 > 0.0f) {  // D / q = 1 - eps_k / q
+    if (d2 > 0.0f) {
       const float l = logf(d2);
-      g.add(t, l);
-      if (P.eps_k > 0.0f) g.add(__fmul_rn(t, -__fdiv_rn(P.eps_k, q)), l);
+      // D / q = 1 - eps_k / q, as long as the quotient is small beside 1: the two parts
+      // cancel otherwise, and its rounding (FP32) would be what is left of them
+      if (P.eps_k <= __fmul_rn(0x1p-7f, D)) {
+        g.add(t, l);
+        if (P.eps_k > 0.0f) g.add(__fmul_rn(t, -__fdiv_rn(P.eps_k, q)), l);
+      } else {
+        gx = __dadd_rn(gx, gamma_term(t, l, D, P.eps_k));
+      }
     }
   }
   __device__ __forceinline__ void store(const LeafArgs &A, uint32_t i, float r2) const {
@@ -577,7 +588,7 @@ struct TrainSums {
     double *const s = A.train.sums + 3ull * i;
     s[0] = w.value();
     s[1] = d.value();
-    s[2] = g.value();
+    s[2] = __dadd_rn(g.value(), gx);
     A.train.r2[i] = r2;
   }
 };
