@@ -715,10 +715,12 @@ uint32_t big_leaf_above(const denoise_params &p, uint32_t n, bool rec) {
 
 int launch_big(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches) {
   const dim3 per_leaf(num_sms), units(num_sms * 2), parts(num_sms * 8);
-  // no leaf is larger than the call: the selects' shared memory
+  // no leaf is larger than the call: the selects' shared memory (their limit is the
+  // same for every call, as other contexts' threads launch the same kernels)
   const size_t sel = 4ull * (a.n < kSelectCap ? a.n : kSelectCap);
-  if (cudaFuncSetAttribute(k_big_gate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel) != cudaSuccess ||
-      cudaFuncSetAttribute(k_big_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel) != cudaSuccess)
+  constexpr int kSelLimit = 4 * (int)kSelectCap;
+  if (cudaFuncSetAttribute(k_big_gate, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelLimit) != cudaSuccess ||
+      cudaFuncSetAttribute(k_big_select, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelLimit) != cudaSuccess)
     return -1;
   launch_pdl(k_big_setup, 1, 1024, 0, st, a);
   launch_pdl(k_big_box, units, kBigUnit, 0, st, a);

@@ -21,6 +21,9 @@ constexpr unsigned long long kInvalid = ~0ull - 1ull;
 constexpr uint32_t kPad = 32;
 // largest leaf of the shared-memory path: bit-sliced counts of the kNN hold < 2^11
 constexpr uint32_t kLeafSmemMax = 2048;
+// Dynamic shared memory a leaf CTA may take (leaf_pick_lmax): the 227 KB of a block less
+// 2 KB for the kernel's static variables.
+constexpr size_t kLeafSmemLimit = 227 * 1024 - 2048;
 
 __host__ __device__ __forceinline__ size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
 // smallest power of two >= x (x <= 2^31; larger x gives 2^31)
@@ -1499,9 +1502,11 @@ __global__ void __launch_bounds__(kNT, leaf_min_ctas(kNT)) k_leaf(const LeafArgs
 template <int kNT, bool kRec, bool kXl>
 inline int launch_k(const LeafArgs &a, int num_sms, cudaStream_t st) {
   const size_t smem = leaf_smem_bytes(a.lmax, a.kmax, kNT);
-  // per call (function attributes are per device, and calls may come from several threads)
-  if (cudaFuncSetAttribute(k_leaf<kNT, kRec, kXl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
+  // The limit belongs to the device's kernel, not to this call, and other contexts'
+  // threads launch the same kernel: always the largest size any call can take.
+  if (smem > kLeafSmemLimit ||
+      cudaFuncSetAttribute(k_leaf<kNT, kRec, kXl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kLeafSmemLimit) != cudaSuccess)
     return -1;
   cudaFuncSetAttribute(k_leaf<kNT, kRec, kXl>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        (int)cudaSharedmemCarveoutMaxShared);
