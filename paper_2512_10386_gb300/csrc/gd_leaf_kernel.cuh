@@ -545,54 +545,132 @@ __device__ __forceinline__ bool rec_index_ok(const LeafArgs &A, uint32_t g) {
 // The sums over a scored point's neighbour terms that the backward pass needs
 // (TrainCache), taken where the neighbours are at hand: keeping the neighbour lists
 // for the backward instead meant 256 scattered bytes a point written and read again.
-// Each sum is an unevaluated pair of floats: products split exactly by a fused
-// multiply-add, additions with their exact rounding error, so it carries what a
-// double-precision sum of the FP32 factors' products does, at FP32 rate.
-struct PairSum {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
-    hi = t;
-    lo = __fadd_rn(lo, __fadd_rn(err, e));
+// They have to carry what FP64 sums of the FP32 factors' exact products do, at FP32
+// rate: the products are split exactly by a fused multiply-add, and each sum is an
+// unevaluated triple of floats whose two upper additions keep their exact rounding
+// error (two sums in the lanes of packed instructions), so a term's error stays below
+// 2^-53 of it.
+struct TripleSum2 {
+  f32x2 s0 = 0, s1 = 0, s2 = 0;
+  static __device__ __forceinline__ f32x2 two_sum(f32x2 &s, f32x2 v) {  // s += v, its rounding error
+    const f32x2 t = add2(s, v), z = sub2(t, s);
+    const f32x2 e = add2(sub2(s, sub2(t, z)), sub2(v, z));
+    s = t;
+    return e;
   }
-  __device__ __forceinline__ double value() const { return __dadd_rn((double)hi, (double)lo); }
+  __device__ __forceinline__ void add(f32x2 v, f32x2 low) {  // v + low, low 2^-20 of v or less
+    const f32x2 e = two_sum(s1, two_sum(s0, v));
+    s2 = add2(s2, add2(e, two_sum(s1, low)));
+  }
+  // the sum of both lanes into the first (FP32: an FP64 instruction costs as much as eight)
+  __device__ __forceinline__ void fold() {
+    auto swap = [](f32x2 v) { return (v >> 32) | (v << 32); };
+    const f32x2 h1 = swap(s0), m1 = swap(s1), l1 = swap(s2);
+    s2 = add2(s2, l1);
+    add(h1, m1);
+  }
+  static __device__ __forceinline__ double value(float h, float m, float l) {
+    return __dadd_rn((double)h, __dadd_rn((double)m, (double)l));
+  }
 };
-// t ln(d^2) D / (D + eps_k) by the definition
-static __device__ __noinline__ double gamma_term(float t, float l, float D, float ek) {
-  return __dmul_rn(__dmul_rn((double)t, (double)l), __ddiv_rn((double)D, __dadd_rn((double)D, (double)ek)));
-}
-struct TrainSums {
-  PairSum w, d, g;
-  double gx = 0.0;
-  __device__ __forceinline__ void add(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
+struct TrainTerm {
+  float t, lw, D, q;  // the term, ln W_ij, (d^2)^(gamma/2), D + eps_k
+  __device__ __forceinline__ TrainTerm(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
     const float lw2 = __fadd_rn(elli, ellj);  // log2 W_ij
-    const float D = g2 ? d2 : exp2f(0.5f * P.gamma * log2f(d2));
-    const float q = __fadd_rn(D, P.eps_k);
-    const float t = __fdiv_rn(exp2f(__fmaf_rn(__fmul_rn(0.5f, P.alpha), lw2, -__fmul_rn(d2, ci))), q);
-    if (t == 0.0f) return;  // (a neighbour of density 0 has ln W = -infinity)
-    w.add(t, __fmul_rn(lw2, 0.6931471805599453f));  // ln W_ij
-    d.add(t, d2);
-    if (d2 > 0.0f) {
-      const float l = logf(d2);
-      // D / q = 1 - eps_k / q, as long as the quotient is small beside 1: the two parts
-      // cancel otherwise, and its rounding (FP32) would be what is left of them
-      if (P.eps_k <= __fmul_rn(0x1p-7f, D)) {
-        g.add(t, l);
-        if (P.eps_k > 0.0f) g.add(__fmul_rn(t, -__fdiv_rn(P.eps_k, q)), l);
-      } else {
-        gx = __dadd_rn(gx, gamma_term(t, l, D, P.eps_k));
-      }
-    }
+    D = g2 ? d2 : exp2f(0.5f * P.gamma * log2f(d2));
+    q = __fadd_rn(D, P.eps_k);
+    t = __fdiv_rn(exp2f(__fmaf_rn(__fmul_rn(0.5f, P.alpha), lw2, -__fmul_rn(d2, ci))), q);
+    lw = __fmul_rn(lw2, 0.6931471805599453f);
   }
-  __device__ __forceinline__ void store(const LeafArgs &A, uint32_t i, float r2) const {
+};
+struct TrainSums {
+  TripleSum2 wd, g;   // (sum t ln W, sum t d^2), and two parts of sum t ln d^2 D / q
+  float near = INFINITY;  // smallest D but 0
+  __device__ __forceinline__ void products(float t, float lw, float d2) {
+    const f32x2 T = pk2(t, t), LW = pk2(lw, d2), p = mul2(T, LW);
+    const float nt = -t;  // fma(-a, b, a b) is minus the product's rounding error
+    wd.add(p, mul2(fma2(pk2(nt, nt), LW, p), pk2(-1.0f, -1.0f)));
+  }
+  // the usual term: eps_k small beside D, so that D / q = 1 - c with c = eps_k / q as
+  // c0 + c1 (q + e = D + eps_k exactly), and products whose splits are exact (see fits)
+  __device__ __forceinline__ void add(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
+    const TrainTerm m(P, g2, d2, elli, ellj, ci);
+    if (m.t == 0.0f) return;  // (a neighbour of density 0 has ln W = -infinity)
+    products(m.t, m.lw, d2);
+    const bool zero = d2 == 0.0f;
+    near = fminf(near, zero ? INFINITY : m.D);
+    const float ek = P.eps_k, l = zero ? 0.0f : logf(d2), gp = __fmul_rn(m.t, l), ge = __fmaf_rn(m.t, l, -gp);
+    const float iq = rcp_hw(m.q), e = __fsub_rn(ek, __fsub_rn(m.q, m.D)), c0 = __fmul_rn(-ek, iq);
+    const float c1 = __fmul_rn(__fsub_rn(__fmaf_rn(-c0, m.q, -ek), __fmul_rn(c0, e)), iq);
+    const float x = __fmul_rn(gp, c0), xe = __fmaf_rn(gp, c0, -x);
+    g.add(pk2(gp, x), pk2(ge, __fadd_rn(xe, __fmaf_rn(gp, c1, __fmul_rn(ge, c0)))));
+  }
+  // Whether every term was a usual one: nothing left the range of FP32 (the sums are
+  // finite), the rounding errors lost below its smallest values are 2^-53 of the sums
+  // or less (F, the sum of t, and sum t d^2 large enough), and eps_k stayed small.
+  __device__ __forceinline__ bool fits(const denoise_params &P, float F) const {
+    float h0, h1, d, w;
+    upk2(wd.s0, w, d);
+    upk2(g.s0, h0, h1);
+    const float none = __fmul_rn(0.0f, __fadd_rn(__fadd_rn(w, d), __fadd_rn(h0, h1)));
+    return none == 0.0f && F >= 0x1p-60f && (d >= 0x1p-90f || d == 0.0f) && P.eps_k <= 0x1p60f &&
+           __fmul_rn(0x1p10f, P.eps_k) <= near;
+  }
+  __device__ __forceinline__ void store(const LeafArgs &A, uint32_t i, float r2) {
     if (!rec_index_ok(A, i)) return;
+    g.fold();
     double *const s = A.train.sums + 3ull * i;
-    s[0] = w.value();
-    s[1] = d.value();
-    s[2] = __dadd_rn(g.value(), gx);
+    float w0, w1, w2, d0, d1, d2, g0, g1, g2, no;
+    upk2(wd.s0, w0, d0);
+    upk2(wd.s1, w1, d1);
+    upk2(wd.s2, w2, d2);
+    upk2(g.s0, g0, no);
+    upk2(g.s1, g1, no);
+    upk2(g.s2, g2, no);
+    s[0] = TripleSum2::value(w0, w1, w2);
+    s[1] = TripleSum2::value(d0, d1, d2);
+    s[2] = TripleSum2::value(g0, g1, g2);
     A.train.r2[i] = r2;
+  }
+};
+// The sums of a point that has other terms too (out of line and apart, which keeps the
+// usual one cheap; 560,000 points, K = 32, leaf stage: 420 us with both in one, 391 so;
+// 365 with pairs of floats, which carry about 48 bits).
+struct TrainSumsAny {
+  TrainSums s;
+  double x[3] = {0.0, 0.0, 0.0};
+  __device__ __noinline__ void add(const denoise_params &P, bool g2, float d2, float elli, float ellj, float ci) {
+    const TrainTerm m(P, g2, d2, elli, ellj, ci);
+    if (m.t == 0.0f) return;
+    const bool zero = d2 == 0.0f;
+    const float t = m.t, D = m.D, q = m.q, ek = P.eps_k, l = logf(d2), td = __fmul_rn(t, d2);
+    // |ln W| and |ln d^2| are below 2^10: beyond these bounds a product's split may not be exact
+    if (!(t >= 0x1p-60f && fmaxf(fmaxf(t, td), D) <= 0x1p110f && (zero || fminf(td, D) >= 0x1p-100f))) {
+      const double T = (double)t;
+      x[0] = __dadd_rn(x[0], __dmul_rn(T, (double)m.lw));
+      x[1] = __dadd_rn(x[1], __dmul_rn(T, (double)d2));
+      if (!zero)
+        x[2] = __dadd_rn(x[2], __dmul_rn(__dmul_rn(T, (double)l), __ddiv_rn((double)D, __dadd_rn((double)D, (double)ek))));
+      return;
+    }
+    s.products(t, m.lw, d2);
+    if (zero) return;
+    // D / q as r0 + r1 + r2 (1 - c would leave c's rounding); r0's remainder is exact
+    const float z = __fsub_rn(q, D), e = __fadd_rn(__fsub_rn(D, __fsub_rn(q, z)), __fsub_rn(ek, z));
+    const float r0 = __fdiv_rn(D, q), a = __fmaf_rn(-r0, q, D), b = __fmul_rn(-r0, e), be = __fmaf_rn(-r0, e, -b);
+    const float rh = __fadd_rn(a, b), y = __fsub_rn(rh, a);
+    const float rl = __fadd_rn(__fsub_rn(a, __fsub_rn(rh, y)), __fsub_rn(b, y));
+    const float r1 = __fdiv_rn(rh, q);
+    const float r2 = __fdiv_rn(__fadd_rn(__fmaf_rn(-r1, q, rh), __fadd_rn(rl, __fmaf_rn(-r1, e, be))), q);
+    const float gp = __fmul_rn(t, l), ge = __fmaf_rn(t, l, -gp);
+    const float x0 = __fmul_rn(gp, r0), x1 = __fmul_rn(gp, r1), w = __fmul_rn(ge, r0);
+    s.g.add(pk2(x0, x1), pk2(__fmaf_rn(gp, r0, -x0), w));
+    s.g.s2 = add2(s.g.s2, pk2(__fmaf_rn(gp, r1, -x1), __fadd_rn(__fmaf_rn(ge, r0, -w), __fmaf_rn(gp, r2, __fmul_rn(ge, r1)))));
+  }
+  __device__ __forceinline__ void store(const LeafArgs &A, uint32_t i, float r2) {
+    if (!rec_index_ok(A, i)) return;
+    s.store(A, i, r2);
+    for (int q = 0; q < 3; ++q) A.train.sums[3ull * i + q] = __dadd_rn(A.train.sums[3ull * i + q], x[q]);
   }
 };
 
@@ -1226,6 +1304,8 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
       const float ai = (train && kPacked) ? __fmul_rn(__fmul_rn(0.5f, P.alpha), M.wa[i]) : M.wa[i];
       float elli = 0.0f;
       TrainSums ts;
+      // (a point whose K-th distance does not stand clear of eps_k is taken term by term at once)
+      const bool any = train && !(__fmul_rn(0x1p14f, ek) <= (g2 ? r2i : pow_half_gamma(r2i, hg)));
       if (train) elli = kPacked ? M.wa[i] : (W[i] < A.n ? A.train.ell[W[i]] : 0.0f);
       // two neighbours per step into two partial sums (independent chains),
       // F = even-rank terms + odd-rank terms
@@ -1239,15 +1319,18 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
       const uint32_t rwords = (n1 + 31u) >> 5;
       const bool cmk_on = !xl && kPacked && n1 <= 1024u;
       // the mask is written by the kNN of this leaf (k_eff > 0); only chunks of the row are taken
-      uint32_t cmk = (cmk_on && keff > 0) ? M.cmask[i] & ((rwords >= 32u) ? 0xFFFFFFFFu : ((1u << rwords) - 1u)) : 0u;
+      uint32_t cmk = 0;
       auto pop_chunk = [&]() -> uint32_t {  // next chunk of the mask (32 if none is left)
         const uint32_t c = cmk ? (uint32_t)(__ffs(cmk) - 1) : 32u;
         cmk &= cmk - 1u;
         return c;
       };
       uint32_t rc = 0, rm = 0, pc = 32, pm = 0;
-      if (kPacked && !xl && keff > 0) {
+      auto rewind = [&]() {  // to the row's first neighbour
+        rc = 0;
+        if (!kPacked || xl || keff == 0) return;
         if (cmk_on) {
+          cmk = M.cmask[i] & ((rwords >= 32u) ? 0xFFFFFFFFu : ((1u << rwords) - 1u));
           rc = pop_chunk();
           rm = rc < 32u ? row[(size_t)rc * n1] : 0u;
           pc = pop_chunk();
@@ -1255,7 +1338,8 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         } else {
           rm = row[0];
         }
-      }
+      };
+      rewind();
       auto next_j = [&](uint32_t t, bool valid) -> uint32_t {  // called for t = 0, 1, ... in order
         if constexpr (kPacked) {
           if (!valid) return 0u;
@@ -1300,12 +1384,24 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
           const float e = __fmul_rn(wt, rcp_hw(__fadd_rn(D, ek)));
           if (t & 1u) F1 = __fadd_rn(F1, e);
           else F0 = __fadd_rn(F0, e);
-          if (train) ts.add(P, g2, d2, elli, __fsub_rn(lj, lsh), ci);
+          if (train && !any) ts.add(P, g2, d2, elli, __fsub_rn(lj, lsh), ci);
         }
         M.F[i] = __fadd_rn(F0, F1);
-        if (train) ts.store(A, W[i], r2i);
+        if (train && (any || !ts.fits(P, M.F[i]))) {
+          TrainSumsAny tx;
+#pragma unroll 1
+          for (uint32_t t = 0; t < keff; ++t) {
+            const float4 pj = A.spts[nl[t]];
+            const float lj = A.xrho ? A.xrho[nl[t]].w : log2_density(A.xkeff[nl[t]], A.xr2[nl[t]]);
+            tx.add(P, g2, sqdist(xi, yi, zi, pj.x, pj.y, pj.z), elli, __fsub_rn(lj, lsh), ci);
+          }
+          tx.store(A, W[i], r2i);
+        } else if (train) {
+          ts.store(A, W[i], r2i);
+        }
         continue;
       }
+      auto ell_of = [&](uint32_t j) { return kPacked ? M.wa[j] : (W[j] < A.n ? A.train.ell[W[j]] : 0.0f); };  // (training)
       // two ranks per step in the two lanes of packed FP32 instructions (even ranks
       // in the low lane, odd in the high: the two partial sums); each lane rounds as
       // the scalar form.  With k_eff odd the last step's second term is computed on
@@ -1338,15 +1434,26 @@ __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__r
         float ta, tb;
         upk2(mul2(pk2(ex2_hw(ea), ex2_hw(eb)), pk2(rcp_hw(qa), rcp_hw(qb))), ta, tb);
         FF = add2(FF, pk2(ta, two ? tb : 0.0f));
-        if (train) {
-          auto ell_of = [&](uint32_t j) { return kPacked ? M.wa[j] : (W[j] < A.n ? A.train.ell[W[j]] : 0.0f); };
-          ts.add(P, g2, da, elli, ell_of(ja), ci);
-          if (two) ts.add(P, g2, db, elli, ell_of(jb), ci);
+        if (train && !any) {
+#pragma unroll 1
+          for (int h = 0; h < (two ? 2 : 1); ++h)  // one copy of the code: instruction fetches
+            ts.add(P, g2, h ? db : da, elli, ell_of(h ? jb : ja), ci);
         }
       }
       upk2(FF, F0, F1);
       M.F[i] = __fadd_rn(F0, F1);
-      if (train) ts.store(A, W[i], r2i);
+      if (train && (any || !ts.fits(P, M.F[i]))) {
+        TrainSumsAny tx;
+        rewind();
+#pragma unroll 1
+        for (uint32_t t = 0; t < keff; ++t) {
+          const uint32_t j = next_j(t, true);
+          tx.add(P, g2, sqdist(xi, yi, zi, X[j], Y[j], Z[j]), elli, ell_of(j), ci);
+        }
+        tx.store(A, W[i], r2i);
+      } else if (train) {
+        ts.store(A, W[i], r2i);
+      }
     }
   }
   __syncthreads();
