@@ -217,7 +217,8 @@ __device__ __forceinline__ float leaf_voxel_size(const float *ext, float delta, 
     const float hh = __fmul_rn(beta, y), hl = __fmaf_rn(beta, c, __fmaf_rn(beta, y, -hh));
     const float eps = __fmul_rn(hh, 0x1p-40f);
     const float lo = __fadd_rn(hh, __fsub_rn(hl, eps)), hi = __fadd_rn(hh, __fadd_rn(hl, eps));
-    if (lo == hi && lo >= 0x1p-60f && lo <= 0x1p60f && k >= -60 && k <= 60) return __fmul_rn(lo, exp2f((float)k));
+    if (lo == hi && lo >= 0x1p-60f && lo <= 0x1p60f && k >= -60 && k <= 60)
+      return __fmul_rn(lo, __int_as_float((127 + k) << 23));  // 2^k from its exponent bits: exact
   }
   return leaf_voxel_size_fp64(H[0], H[1], H[2], count, beta);
 }
