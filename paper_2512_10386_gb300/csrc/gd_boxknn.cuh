@@ -360,11 +360,15 @@ __device__ __forceinline__ bool bk_knn(const Src &src, BkShared<KROW> &S, bool a
   f32x2 QX = pk2(qx, qx), QY = pk2(qy, qy), QZ = pk2(qz, qz);
   Box qb = box_warp_union(box_point(qx, qy, qz));
   far = 0;
-  // theta_0: outward from q until k valid others are seen
+  // theta_0: outward from q until k valid others are seen, but no further than where a
+  // candidate in sixteen positions would have done: each step waits for its loads, and
+  // where the voxel gate left few points of a large leaf the walk would cross it (one leaf
+  // of 1 M points, 200 of them candidates, K = 32: 46.9 -> 1.5 ms)
   float t0 = 0.0f;
   {
     uint32_t found = 0;
-    for (uint32_t d = 1; __any_sync(0xFFFFFFFFu, found < k && (q >= w0 + d || q + d < w1)); ++d) {
+    const uint32_t steps = 8u * k + 32u;
+    for (uint32_t d = 1; d <= steps && __any_sync(0xFFFFFFFFu, found < k && (q >= w0 + d || q + d < w1)); ++d) {
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const bool in = found < k && (side ? q + d < w1 : q >= w0 + d);
@@ -379,8 +383,8 @@ __device__ __forceinline__ bool bk_knn(const Src &src, BkShared<KROW> &S, bool a
       }
     }
     if (__any_sync(0xFFFFFFFFu, found < k)) {
-      // too few points around the query: no candidate lies beyond the far corner of
-      // its super-chunk's box
+      // too few points around the query: no candidate lies beyond the far corners of
+      // the super-chunks' boxes
       const Box me = box_point(qx, qy, qz);
       float far = 0.0f;
       for (uint32_t e = 0; e < src.entries(); ++e) {
