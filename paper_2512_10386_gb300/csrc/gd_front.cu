@@ -986,6 +986,52 @@ __device__ __forceinline__ void small_order(const unsigned long long *full, unsi
   __syncthreads();
 }
 
+// One more sort of the positions: inside a big node by the key bits below it (at most 33:
+// key_low to sh) and the input index, elsewhere by the position itself.  Both ends of
+// an item's node are searched (the order is by node), and the sort is the registers' again:
+// 4,096 points of which all but one share a node, capacity 1,024: front end 478 us with
+// members counted one by one and a comparison network over buf, 104 so.
+template <int E>
+__device__ __forceinline__ void small_nodes(const unsigned long long *full, unsigned long long *buf, uint32_t n,
+                                            uint32_t cap, int sh, int key_low) {
+  static_assert(kSmallFront <= 1u << 12, "positions and indices in 12 bits each");
+  const uint32_t t = threadIdx.x;
+  unsigned long long v[E];
+  uint32_t a = 0, b = 0;  // positions [a, b): the node of the thread's last item
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const uint32_t p = t * E + k;
+    v[k] = ~0ull;
+    if (p >= n) continue;
+    const uint32_t idx = (uint32_t)buf[p];
+    const unsigned long long key = full[idx], pre = key >> sh;
+    if (p >= b) {
+      a = b;
+      b = n;
+      for (uint32_t hi = p; a < hi;) {
+        const uint32_t mid = (a + hi) >> 1;
+        if (full[(uint32_t)buf[mid]] >> sh == pre) hi = mid;
+        else a = mid + 1u;
+      }
+      for (uint32_t lo = p + 1u; lo < b;) {
+        const uint32_t mid = (lo + b) >> 1;
+        if (full[(uint32_t)buf[mid]] >> sh == pre) lo = mid + 1u;
+        else b = mid;
+      }
+    }
+    const unsigned long long low = (key & ((1ull << sh) - 1ull)) >> key_low;
+    v[k] = b - a > cap ? ((unsigned long long)a << 45) | (low << 12) | idx : ((unsigned long long)p << 45) | idx;
+  }
+  uint32_t N = 2;
+  while (N < n) N <<= 1;
+  __syncthreads();
+  small_sort<E>(v, buf, N);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < E; ++k) buf[t * E + k] = v[k] & 0xFFFull;
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kSmallThreads) k_front_small(const SmallArgs A) {
   extern __shared__ unsigned long long s_dyn[];
   unsigned long long *const full = s_dyn, *const buf = s_dyn + kSmallFront;  // keys by input index; order
@@ -1078,46 +1124,16 @@ __global__ void __launch_bounds__(kSmallThreads) k_front_small(const SmallArgs A
   } else {
     small_order<4>(full, buf, n, A.lowbit);
   }
-  // ---- the big level-DB nodes in full octree order (rare): one more network over all
-  // items, which outside those nodes compares what it did before
+  // ---- the big level-DB nodes in full octree order (rare)
   if (A.DB < A.D) {
     const int sh = 63 - 3 * A.DB;
-    auto key_at = [&](uint32_t p) { return full[(uint32_t)buf[p] & 0x7FFFFFFFu]; };  // (the flag set below)
+    auto node = [&](uint32_t p) { return full[(uint32_t)buf[p]] >> sh; };
     bool any = false;
-    for (uint32_t i = tid; i < n; i += kSmallThreads) any |= n - i > A.cap && (key_at(i) >> sh) == (key_at(i + A.cap) >> sh);
+    for (uint32_t i = tid; i < n; i += kSmallThreads) any |= n - i > A.cap && node(i) == node(i + A.cap);
     if (__syncthreads_or(any)) {
-      uint32_t N = 2;
-      while (N < n) N <<= 1;
-      // an item's sort key: everything in a big node, the sorted bits elsewhere
-      auto skey = [&](uint32_t idx, bool big) { return big ? full[idx] >> A.key_low : (full[idx] >> A.lowbit) << (A.lowbit - A.key_low); };
-      for (uint32_t i = tid; i < n; i += kSmallThreads) {
-        const unsigned long long pre = key_at(i) >> sh;
-        uint32_t a = i, b = i + 1;
-        while (a > 0 && i - a <= A.cap && (key_at(a - 1) >> sh) == pre) --a;
-        while (b < n && b - a <= A.cap && (key_at(b) >> sh) == pre) ++b;
-        // the flag travels in the top bit of the index word
-        if (b - a > A.cap) atomicOr(reinterpret_cast<uint32_t *>(buf) + 2 * i, 0x80000000u);
-      }
-      __syncthreads();
-      for (uint32_t size = 2; size <= N; size <<= 1) {
-        for (uint32_t j = size >> 1; j > 0; j >>= 1) {
-          for (uint32_t c = tid; c < (N >> 1); c += kSmallThreads) {
-            const uint32_t a = 2 * j * (c / j) + (c % j), b = a + j;
-            const bool up = (a & size) == 0;
-            const uint32_t ia = (uint32_t)buf[a], ib = (uint32_t)buf[b];
-            // the padding (all ones) sorts last
-            const unsigned long long ka = buf[a] == ~0ull ? ~0ull : skey(ia & 0x7FFFFFFFu, ia >> 31);
-            const unsigned long long kb = buf[b] == ~0ull ? ~0ull : skey(ib & 0x7FFFFFFFu, ib >> 31);
-            const bool less = kb < ka || (kb == ka && (ib & 0x7FFFFFFFu) < (ia & 0x7FFFFFFFu));
-            if (less == up) {
-              const unsigned long long x0 = buf[a];
-              buf[a] = buf[b];
-              buf[b] = x0;
-            }
-          }
-          __syncthreads();
-        }
-      }
+      if (n <= kSmallThreads) small_nodes<1>(full, buf, n, A.cap, sh, A.key_low);
+      else if (n <= 2 * kSmallThreads) small_nodes<2>(full, buf, n, A.cap, sh, A.key_low);
+      else small_nodes<4>(full, buf, n, A.cap, sh, A.key_low);
     }
   }
   // ---- results in order; then the sorted keys take the order's place.  (Host input is
@@ -1128,7 +1144,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_front_small(const SmallArgs A
   for (int k = 0; k < kSmallItems; ++k) {
     const uint32_t i = (uint32_t)k * kSmallThreads + tid;
     if (i < n) {
-      const uint32_t v = (uint32_t)buf[i] & 0x7FFFFFFFu;
+      const uint32_t v = (uint32_t)buf[i];
       sk[k] = full[v];
       A.keys[i] = sk[k];
       A.spts[i] = make_float4(src[3ull * v], src[3ull * v + 1], src[3ull * v + 2], __uint_as_float(v));
