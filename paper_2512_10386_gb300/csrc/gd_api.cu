@@ -86,7 +86,7 @@ struct denoise_ctx {
   // frame layout cache
   std::vector<uint64_t> layout;
   uint32_t ntiles = 0;
-  uint32_t frame_tiles = 0;       // of the largest frame
+  uint32_t frame_tiles = 0, frame_points = 0;  // of the largest frame
   uint64_t layout_gen = 0;        // bumped at every layout change
   uint64_t tables_gen = ~0ull;    // layout generation that d_tiles / d_frames hold (after a direct call)
 };
@@ -195,7 +195,7 @@ int map_status(uint32_t st) {
 // Front-end tiles of a frame layout (host); returns the tile count.
 uint32_t build_tiles(denoise_ctx *c, const uint64_t *offsets, uint32_t nframes) {
   uint32_t nt = 0;
-  c->frame_tiles = 0;
+  c->frame_tiles = c->frame_points = 0;
   for (uint32_t f = 0; f < nframes; ++f) {
     const uint32_t b = (uint32_t)offsets[f], e = (uint32_t)offsets[f + 1];
     FrameInfo &fi = c->h_frames[c->slot][f];
@@ -208,6 +208,7 @@ uint32_t build_tiles(denoise_ctx *c, const uint64_t *offsets, uint32_t nframes) 
       c->h_tiles[c->slot][nt++] = Tile{f, s, te, first};
     }
     if (nt - first > c->frame_tiles) c->frame_tiles = nt - first;
+    if (e - b > c->frame_points) c->frame_points = e - b;
   }
   return nt;
 }
@@ -261,7 +262,11 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   la.spin_limit = c->wait_limit;
   const int kmax = leaf_kmax(p.k);
   la.kmax = kmax;
-  la.lmax = leaf_pick_lmax(p.leaf_capacity, kmax, c->smem_optin - 2048);
+  // no leaf is larger than the largest frame: a batch of small frames has the layout and
+  // the CTA width of their size (3,000 frames of 20 points at capacity 512, leaf stage:
+  // 248 us with 512 threads a leaf, 47 so)
+  la.lmax = leaf_pick_lmax(p.leaf_capacity < c->frame_points ? p.leaf_capacity : c->frame_points, kmax,
+                           c->smem_optin - 2048);
   if (const uint32_t above = big_leaf_above(p, n, dbg != nullptr || c->training != 0)) {
     la.skip_big = 1;
     la.unit_start = c->d_vals[0];  // free after the front end, as the other key buffer

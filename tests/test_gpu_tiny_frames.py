@@ -1,0 +1,65 @@
+"""Batches of small frames under a large leaf capacity: results of each frame's own call,
+and a leaf stage as fast as under a capacity of the frames' size.
+
+Tolerance of the time: the capacity may make the stage half as long again."""
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _cloud(n, seed):
+    g = torch.Generator().manual_seed(seed)
+    v = torch.randn(n, 3, generator=g)
+    return (v / v.norm(dim=1, keepdim=True) + 0.01 * torch.randn(n, 3, generator=g)).cuda()
+
+
+@pytest.mark.parametrize("sizes", [[1, 2, 20, 64, 65, 3], [128, 129, 40, 0, 256], [257, 5, 600], [1500, 30, 700]])
+@pytest.mark.parametrize("cap", [16, 64, 512, 2048, 0xFFFFFFFF])
+def test_frames_alone_and_together(sizes, cap):
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2512_10386_gb300 import Denoiser, Params
+    parts = [_cloud(n, 7 * n + i) for i, n in enumerate(sizes)]
+    offs = [0]
+    for p in parts:
+        offs.append(offs[-1] + len(p))
+    d = Denoiser(max_points=offs[-1], max_frames=len(parts))
+    try:
+        P = Params(k=8, leaf_capacity=cap, min_vox_count=2)
+        b = d.run_batch(torch.cat(parts), offs, P)
+        for f, p in enumerate(parts):
+            if len(p) == 0:
+                continue
+            r = d.run_debug(p, P)
+            for a, c in ((r["mask"], b.mask), (r["stage"], b.stage), (r["score"], b.score)):
+                assert torch.equal(a, c[offs[f]:offs[f + 1]])
+    finally:
+        d.close()
+
+
+def _stage(frames, m, cap, stage):
+    from paper_2512_10386_gb300 import Denoiser, Params
+    x = _cloud(frames * m, 3)
+    offs = [i * m for i in range(frames + 1)]
+    d = Denoiser(max_points=len(x), max_frames=frames)
+    try:
+        d.set_profiling(True)
+        t = []
+        for _ in range(12):
+            d.run_batch(x, offs, Params(k=8, leaf_capacity=cap))
+            t.append(d.stats()["stage_ms"][stage])
+        return sorted(t)[6]
+    finally:
+        d.close()
+
+
+@pytest.mark.parametrize("m", [20, 100])
+def test_leaf_stage_of_small_frames(m):
+    import __graft_entry__
+    __graft_entry__.build()
+    small, large = _stage(3000, m, 64 if m == 20 else 128, 4), _stage(3000, m, 512, 4)
+    print(small, large)
+    assert large <= 1.5 * small, (small, large)
