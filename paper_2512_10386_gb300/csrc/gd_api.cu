@@ -86,7 +86,7 @@ struct denoise_ctx {
   // frame layout cache
   std::vector<uint64_t> layout;
   uint32_t ntiles = 0;
-  uint32_t frame_tiles = 0, frame_points = 0;  // of the largest frame
+  uint32_t frame_points = 0;      // of the largest frame
   uint64_t layout_gen = 0;        // bumped at every layout change
   uint64_t tables_gen = ~0ull;    // layout generation that d_tiles / d_frames hold (after a direct call)
 };
@@ -195,7 +195,7 @@ int map_status(uint32_t st) {
 // Front-end tiles of a frame layout (host); returns the tile count.
 uint32_t build_tiles(denoise_ctx *c, const uint64_t *offsets, uint32_t nframes) {
   uint32_t nt = 0;
-  c->frame_tiles = c->frame_points = 0;
+  c->frame_points = 0;
   for (uint32_t f = 0; f < nframes; ++f) {
     const uint32_t b = (uint32_t)offsets[f], e = (uint32_t)offsets[f + 1];
     FrameInfo &fi = c->h_frames[c->slot][f];
@@ -207,7 +207,6 @@ uint32_t build_tiles(denoise_ctx *c, const uint64_t *offsets, uint32_t nframes) 
       const uint32_t te = (e - s > (uint32_t)kTilePts) ? s + kTilePts : e;
       c->h_tiles[c->slot][nt++] = Tile{f, s, te, first};
     }
-    if (nt - first > c->frame_tiles) c->frame_tiles = nt - first;
     if (e - b > c->frame_points) c->frame_points = e - b;
   }
   return nt;
@@ -291,7 +290,7 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   fa.nframes = nframes;
   fa.tiles = c->d_tiles;
   fa.ntiles = c->ntiles;
-  fa.frame_tiles = c->frame_tiles;
+  fa.frame_points = c->frame_points;
   fa.keys[0] = c->d_keys[0];
   fa.keys[1] = c->d_keys[1];
   fa.vals[0] = c->d_vals[0];

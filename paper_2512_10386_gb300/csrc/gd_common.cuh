@@ -186,7 +186,7 @@ struct FrontArgs {
   uint32_t nframes;
   const Tile *tiles;
   uint32_t ntiles;
-  uint32_t frame_tiles;   // of the largest frame
+  uint32_t frame_points;  // of the largest frame
   unsigned long long *keys[2];
   uint32_t *vals[2];
   float4 *spts;

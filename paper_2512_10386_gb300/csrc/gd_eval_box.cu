@@ -556,7 +556,7 @@ int eb_build(const EbMem &m, const float *a, uint32_t na, const float *b, uint32
   f.nframes = nb ? 2 : 1;
   f.tiles = m.tiles;
   f.ntiles = (na + kTilePts - 1) / kTilePts + (nb + kTilePts - 1) / kTilePts;
-  f.frame_tiles = ((na > nb ? na : nb) + kTilePts - 1) / kTilePts;
+  f.frame_points = na > nb ? na : nb;
   for (int i = 0; i < 2; ++i) {
     f.keys[i] = m.keys[i];
     f.vals[i] = m.vals[i];

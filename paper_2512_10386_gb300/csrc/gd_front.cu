@@ -793,7 +793,17 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
   __shared__ uint32_t s_wsum[kFrontThreads / 32];
   __shared__ uint32_t s_base;
   __shared__ uint32_t s_sh[3][kLeavesWords];  // bytes: shared() + 1 (0: none) from position t.begin - cap on; window maxima
-  if (cap <= kLeavesSmemCap) {  // block-uniform
+  if (fe - fb <= cap || t.begin >= t.end) {
+    // the frame is one leaf (the root: level 0), or the tile ends before this part: no keys
+    // are needed (3,000 frames of 20 points under a capacity of 512: 55 us with the window's
+    // passes in every block, 20 so)
+#pragma unroll
+    for (int it = 0; it < kLeavesItems; ++it) s_cnt[it][threadIdx.x] = 0;
+    if (t.begin == fb && t.begin < t.end && threadIdx.x == 0) {
+      s_cnt[0][0] = fe - fb;
+      s_lvl[0][0] = 0;
+    }
+  } else if (cap <= kLeavesSmemCap) {  // (all block-uniform)
     const uint32_t wb = (t.begin - fb > cap + 1) ? t.begin - cap - 1 : fb;
     const uint32_t we = (fe - t.end > cap + 1) ? t.end + cap + 1 : fe;
     for (uint32_t i = wb + threadIdx.x; i < we; i += kFrontThreads) s_win[i - wb] = keys[i];
@@ -1224,7 +1234,7 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
   }
   const InitArgs init{a.nframes, a.ctr, a.digit_hist, a.lookback, nlb, passes};
   launch_pdl(k_bbox, a.ntiles, kFrontThreads, 0, st, a.xyz_src ? a.xyz_src : a.xyz, a.xyz_copy, a.tile_box, a.tiles, init);
-  if (a.frame_tiles > kBoxTiles) {
+  if (a.frame_points > kBoxTiles * (uint32_t)kTilePts) {
     launch_pdl(k_frame_box, (a.ntiles + kBoxTiles - 1) / kBoxTiles, 1024, 0, st, a.tile_box, a.tiles, a.frames);
     ++nl;
   }
@@ -1267,7 +1277,8 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
     ++nl;
   }
   if (ev_after_sort) cudaEventRecord(*ev_after_sort, st);
-  const size_t win = (a.leaf_capacity <= kLeavesSmemCap)
+  // (no window where every frame is one leaf)
+  const size_t win = (a.leaf_capacity <= kLeavesSmemCap && a.frame_points > a.leaf_capacity)
                         ? sizeof(unsigned long long) * (kLeavesPart + 2 * ((size_t)a.leaf_capacity + 1))
                         : 0;
   if (cudaFuncSetAttribute(k_leaves, cudaFuncAttributeMaxDynamicSharedMemorySize,

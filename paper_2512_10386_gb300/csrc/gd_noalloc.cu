@@ -156,6 +156,7 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
   fa.nframes = 1;
   fa.tiles = tiles;
   fa.ntiles = ntiles;
+  fa.frame_points = nn;
   fa.keys[0] = (unsigned long long *)(b + kOffKeys0);
   fa.keys[1] = (unsigned long long *)(b + kOffKeys1);
   fa.vals[0] = (uint32_t *)(b + kOffVals0);

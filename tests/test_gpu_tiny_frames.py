@@ -63,3 +63,12 @@ def test_leaf_stage_of_small_frames(m):
     small, large = _stage(3000, m, 64 if m == 20 else 128, 4), _stage(3000, m, 512, 4)
     print(small, large)
     assert large <= 1.5 * small, (small, large)
+
+
+def test_leaf_finder_of_small_frames():
+    import __graft_entry__
+    __graft_entry__.build()
+    # under a capacity of 8 the finder searches every frame, above 20 there is nothing to search
+    search, whole = _stage(3000, 20, 8, 2), _stage(3000, 20, 2048, 2)
+    print(search, whole)
+    assert whole <= search, (search, whole)
