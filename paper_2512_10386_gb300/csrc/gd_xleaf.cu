@@ -17,7 +17,7 @@
 // For K <= 32 the P_1 points get chunk boxes (k_xleaf_boxes), every leaf its 27 ranges
 // and |C_t| once (k_xleaf_ranges), and one warp finds the neighbours of 32 queries by
 // counting, reading only the chunks of the ranges that can hold one (gd_boxknn.cuh;
-// k_xleaf_knn_box, k_xleaf_knn_far).  A 560,000-point scan, K = 32: 3.2 G pairs in the
+// k_xleaf_knn_box, k_xleaf_knn_far; small calls: k_xleaf_knn_far alone).  A 560,000-point scan, K = 32: 3.2 G pairs in the
 // ranges, 8.5 ms with every candidate compared, 3.0 ms so (1.7 the box search, 0.8 the
 // far queries), bound by instruction issue.  Larger K keep the per-thread list (k_xleaf_knn).
 #include <cuda_runtime.h>
@@ -217,10 +217,7 @@ __global__ void __launch_bounds__(1024) k_xleaf_units(const Leaf *__restrict__ l
     if (tid == 1023) s_run = run + s_w[w] + inc;
     __syncthreads();
   }
-  if (tid == 0) {
-    ctr->x_units = s_run;
-    ctr->far_count = 0;
-  }
+  if (tid == 0) ctr->x_units = s_run;
 }
 
 // A leaf's candidate ranges, at the start of its slice of the spill area (idle
@@ -241,6 +238,7 @@ __global__ void __launch_bounds__(kBoxSuper) k_xleaf_boxes(const XleafArgs A) {
   if (A.ctr->status & kStFatal) return;
   const BoxIndex bx = box_index(A.boxes, A.n);
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, i = blockIdx.x * kBoxSuper + threadIdx.x;
+  if (i == 0) A.ctr->far_count = 0;
   Box b = box_empty();
   const bool in = i < A.n && A.xflag[i];
   if (in) {
@@ -263,8 +261,15 @@ __global__ void __launch_bounds__(kBoxSuper) k_xleaf_boxes(const XleafArgs A) {
   }
 }
 
-// the 27 ranges of every leaf and |C_t|: one warp a leaf
-__global__ void __launch_bounds__(128) k_xleaf_ranges(const XleafArgs A) {
+// Calls of at most this many points give every query a warp of its own at once: they have
+// too few warps of 32 queries to fill the GPU, and each is a chain of four passes.  us a
+// call, warps of 32 queries / of one (K = 12, leaves of 64; K = 32, 256): 1,500 points 265 / 158,
+// 271 / 160; 6,000 327 / 212, 387 / 237; 10,000 347 / 224, 488 / 272.
+constexpr uint32_t kXSmall = 16384;
+
+// the 27 ranges of every leaf and |C_t|: one warp a leaf; with `queue` its queries too go
+// on the list of those with a warp of their own
+__global__ void __launch_bounds__(128) k_xleaf_ranges(const XleafArgs A, const bool queue) {
   pdl_wait();
   if (A.ctr->status & kStFatal) return;
   const uint32_t lane = threadIdx.x & 31u, nl = A.ctr->n_leaves;
@@ -311,6 +316,24 @@ __global__ void __launch_bounds__(128) k_xleaf_ranges(const XleafArgs A) {
       x->rng[lane][1] = b;
     }
     if (lane == 0) x->nc = cnt;
+    if (queue) {
+      uint32_t nq = 0;
+      for (uint32_t q0 = 0; q0 < lf.count; q0 += 32u) {
+        const uint32_t q = lf.start + q0 + lane;
+        const bool act = q0 + lane < lf.count && A.xflag[q];
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, act);
+        if (!m) continue;
+        uint32_t slot = 0;
+        if (lane == 0) slot = atomicAdd(&A.ctr->far_count, (uint32_t)__popc(m));
+        slot = __shfl_sync(0xFFFFFFFFu, slot, 0) + __popc(m & lanemask_lt());
+        if (act) {
+          A.far_queue[slot] = make_uint2(li, q);
+          A.xr2[q] = INFINITY;  // no bound yet
+        }
+        nq += __popc(m);
+      }
+      if (lane == 0 && nq && cnt > 1) atomicAdd(&A.ctr->knn_pairs, (unsigned long long)nq * (cnt - 1));
+    }
   }
 }
 
@@ -481,7 +504,11 @@ __global__ void __launch_bounds__(128) k_xleaf_knn_far(const XleafArgs A) {
     const uint2 e = A.far_queue[i];
     const Leaf lf = A.leaves[e.x];
     const XRanges *const xr = x_ranges(A, lf);
-    const uint32_t nc = xr->nc, keff = A.k < nc - 1 ? A.k : nc - 1;
+    const uint32_t nc = xr->nc, keff = nc <= 1 ? 0u : A.k < nc - 1 ? A.k : nc - 1;
+    if (keff == 0) {  // alone in its block of cells
+      x_emit<kRec>(A, e.y, 0u, 0ull, 0u, 0.f, lane);
+      continue;
+    }
     x_load(X, xr, lane);
     const float4 me = A.spts[e.y];
     const XSrc src{A.spts, A.xflag, bx, X.rng, X.off};
@@ -500,11 +527,12 @@ int launch_x(const XleafArgs &a, int num_sms, cudaStream_t st, int *launches) {
   cudaError_t e;
   if (a.k <= 32) {
     e = launch_pdl(k_xleaf_boxes, box_supers(a.n), kBoxSuper, 0, st, a);
-    if (e == cudaSuccess) e = launch_pdl(k_xleaf_units, 1, 1024, 0, st, a.leaves, a.ctr, a.unit_start);
-    if (e == cudaSuccess) e = launch_pdl(k_xleaf_ranges, num_sms * 8, 128, 0, st, a);
-    if (e == cudaSuccess) e = launch_pdl(k_xleaf_knn_box<kRec>, num_sms * 6, 32 * kBkWarps, 0, st, a);
+    const bool small = a.n <= kXSmall;
+    if (e == cudaSuccess && !small) e = launch_pdl(k_xleaf_units, 1, 1024, 0, st, a.leaves, a.ctr, a.unit_start);
+    if (e == cudaSuccess) e = launch_pdl(k_xleaf_ranges, num_sms * 8, 128, 0, st, a, small);
+    if (e == cudaSuccess && !small) e = launch_pdl(k_xleaf_knn_box<kRec>, num_sms * 6, 32 * kBkWarps, 0, st, a);
     if (e == cudaSuccess) e = launch_pdl(k_xleaf_knn_far<kRec>, num_sms * 8, 128, 0, st, a);
-    if (launches) *launches += 5;
+    if (launches) *launches += small ? 3 : 5;
   } else {
     e = go(k_xleaf_knn<64, kRec>);
     if (launches) *launches += 1;
