@@ -41,6 +41,12 @@ constexpr uint32_t kQuarter = kBoxChunk / 4;
 __device__ __forceinline__ bool cnt_apart(uint32_t listed, uint32_t own) {
   return listed * 190u > 32u * (600u + 15u * own);
 }
+// Below this many chunks of queries the warps of a block share one, each with a fourth of
+// the super-chunks: one warp a chunk leaves most of the GPU's schedulers one warp or
+// two, waiting for their own loads.  us a call, one / four warps, R = 0.05 / 0.45 of the
+// extent: 36,750 points of a sphere 245 / 205, 824 / 448 (the full pass 540); 200,000 399 /
+// 369, 4407 / 2694; 560,000 at 0.02 / 0.3 589 / 651, 7039 / 6211; 1 M 1058 / 1280, 16610 / 15684.
+constexpr uint32_t kCntSplit = 8192;
 constexpr float kInf = INFINITY;
 
 struct Cloud {                  // one cloud in octree order
@@ -384,17 +390,28 @@ __device__ __forceinline__ uint32_t eb_border(const Cloud &C, EbChunk &S, const 
   return beyond;
 }
 
+// kSplit warps (1 or all of a block) share a chunk of queries, each with every kSplit-th
+// super-chunk.
+template <int kSplit>
 __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const float *__restrict__ r2_dev,
                                                           uint32_t *__restrict__ out, uint32_t *__restrict__ far,
                                                           EbWork *work, const Counters *ctr) {
+  static_assert(kSplit == 1 || kSplit == kEbWarps, "the warps of a chunk are one warp or the whole block");
   __shared__ __align__(16) EbChunk s_c[kEbWarps];
   __shared__ uint32_t s_list[kEbWarps][kCntList], s_part[kEbWarps][4u * kCntBlock + 3u];
+  __shared__ uint32_t s_sum[2], s_out[kBoxChunk];
   if (ctr->status & kStFatal) return;
-  EbChunk &S = s_c[threadIdx.x >> 5];
-  uint32_t *const list = s_list[threadIdx.x >> 5], *const part = s_part[threadIdx.x >> 5];
+  const uint32_t w = threadIdx.x >> 5, share = w % kSplit;
+  EbChunk &S = s_c[w];
+  uint32_t *const list = s_list[w], *const part = s_part[w];
   const uint32_t lane = threadIdx.x & 31u, nsu = box_supers(C.n), nch = box_chunks(C.n);
-  const uint32_t qc = blockIdx.x * kEbWarps + (threadIdx.x >> 5);
+  const uint32_t qc = (blockIdx.x * kEbWarps + w) / kSplit;
   if (qc >= nch) return;
+  if (kSplit > 1) {
+    if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
+    if (threadIdx.x < kBoxChunk) s_out[threadIdx.x] = 0;
+    __syncthreads();
+  }
   const float r2 = *r2_dev;
   const uint32_t q = qc * kBoxChunk + lane;
   const float4 me = C.pts[q < C.n ? q : C.n - 1u];
@@ -407,12 +424,14 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
   // counts those that one of the queries needs, to see whether the queries belong
   // together; a second one runs where they do and the list was too short for all.
   uint32_t whole = 0, beyond = 0, done = 0, nl = 0, own = 0;
+  const uint32_t mine = kSplit > 1 ? 0x11111111u << share : 0xFFFFFFFFu;  // lanes: this warp's super-chunks
+  static_assert(kEbWarps == 4, "the mask of a fourth");
 #pragma unroll 1
   for (int round = 0; round < 2; ++round) {
     for (uint32_t s0 = 0; s0 < nsu; s0 += 32u) {
       const uint32_t s = s0 + lane;
       bool in = false, edge = false;
-      if (s < nsu) {
+      if (s < nsu && ((mine >> lane) & 1u)) {
         const Box sb = box_load(C.box.super, s);
         in = box_upper(sb, qb) <= r2;
         edge = !in && box_lower(sb, qb) <= r2;
@@ -443,8 +462,18 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
       }
     }
     if (round == 0) {
-      if (cnt_apart(nl, own)) {
-        if (lane == 0) far[atomicAdd(&work->cnt_far, 1u)] = qc;
+      uint32_t listed = nl;
+      if (kSplit > 1) {
+        if (lane == 0) {
+          atomicAdd(&s_sum[0], nl);
+          atomicAdd(&s_sum[1], own);
+        }
+        __syncthreads();
+        listed = s_sum[0];
+        own = s_sum[1];
+      }
+      if (cnt_apart(listed, own)) {
+        if (lane == 0 && share == 0) far[atomicAdd(&work->cnt_far, 1u)] = qc;
         return;
       }
       if (nl <= kCntList) break;
@@ -453,8 +482,14 @@ __global__ void __launch_bounds__(kEbThreads) k_evb_count(const Cloud C, const f
     }
   }
   beyond += eb_border(C, S, list, nl, part, qb, r2, QX, QY, QZ, R2, whole, done);
-  whole = __reduce_add_sync(0xFFFFFFFFu, whole);
-  if (q < C.n) out[__float_as_uint(me.w) - C.first] = whole + done * kBoxChunk - beyond;
+  uint32_t cnt = __reduce_add_sync(0xFFFFFFFFu, whole) + done * kBoxChunk - beyond;
+  if (kSplit > 1) {
+    atomicAdd(&s_out[lane], cnt);
+    __syncthreads();
+    if (share != 0) return;
+    cnt = s_out[lane];
+  }
+  if (q < C.n) out[__float_as_uint(me.w) - C.first] = cnt;
 }
 
 // the chunks of queries that lie far apart: one query a warp
@@ -611,8 +646,11 @@ int launch_evb_count(unsigned char *scratch, const float *xyz, uint32_t n, const
   eb_carve(scratch, n, 0, &m);
   Cloud c[2];
   if (eb_build(m, xyz, n, nullptr, 0, ctr, spin_limit, num_sms, c, st)) return -1;
-  k_evb_count<<<(box_chunks(n) + kEbWarps - 1) / kEbWarps, kEbThreads, 0, st>>>(
-      c[0], r2_dev, cnt, m.vals[0], m.work, ctr);
+  if (box_chunks(n) < kCntSplit)
+    k_evb_count<kEbWarps><<<box_chunks(n), kEbThreads, 0, st>>>(c[0], r2_dev, cnt, m.vals[0], m.work, ctr);
+  else
+    k_evb_count<1><<<(box_chunks(n) + kEbWarps - 1) / kEbWarps, kEbThreads, 0, st>>>(c[0], r2_dev, cnt, m.vals[0],
+                                                                                      m.work, ctr);
   k_evb_count_far<<<num_sms * 8, kEbThreads, 0, st>>>(c[0], r2_dev, cnt, m.vals[0], m.work, ctr);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
