@@ -28,8 +28,14 @@ constexpr int kEbThreads = 32 * kEbWarps;
 // costs the warp about 200 instructions, a query of its own about 700.  With fewer
 // warps than fill the GPU the last warp's time counts, and queries leave earlier.
 // Measured, us a call at shares 1 / 2 / 4: object of 30,000 points 266 / 308 / 334,
-// scans of 250,000 709 / 609 / 608 and 500,000 1499 / 1075 / 946.
-inline float nn_share(uint32_t chunks) { return chunks < 2500u ? 1.0f : chunks < 8000u ? 2.0f : 4.0f; }
+// scans of 250,000 709 / 609 / 608 and 500,000 1499 / 1075 / 946.  A cloud of a few
+// hundred chunks of queries (against one of millions of points) has too few warps for
+// anything else: each query leaves at its first chunk.  us a call, share 1 / 0 (the full
+// pass): 500 against 1.2 M uniform points 604 / 400 (430), 1,600 against 400,000 397 / 265
+// (386), 16,000 against 1.2 M 618 / 518 (7187).
+inline float nn_share(uint32_t chunks) {
+  return chunks < 600u ? 0.0f : chunks < 2500u ? 1.0f : chunks < 8000u ? 2.0f : 4.0f;
+}
 constexpr uint32_t kCntList = 768;   // chunks of the radius count's list
 constexpr uint32_t kCntBlock = 64;   // of them split into quarters at a time
 constexpr uint32_t kQuarter = kBoxChunk / 4;
