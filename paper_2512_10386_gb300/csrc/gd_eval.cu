@@ -426,9 +426,14 @@ int launch_eval_metrics(const EvalArgs &e, int num_sms, cudaStream_t st) {
   double *red = (double *)take(8ull * 9 * ra);
   double *pa_sum = (double *)take(8ull * ra), *pb_sum = (double *)take(8ull * rb);
   const FrameInfo *frame = nullptr;
+  bool direct = false;
   if (e.box_scratch) {
-    if (e.nn_clean) da = reinterpret_cast<uint32_t *>(e.nn_clean);  // the distances go where the caller wants them
-    if (e.nn_denoised) db = reinterpret_cast<uint32_t *>(e.nn_denoised);
+    // the distances go where the caller wants them, unless one output lies over the other
+    // (the sums below read both)
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(e.nn_clean), b0 = reinterpret_cast<uintptr_t>(e.nn_denoised);
+    direct = !(a0 && b0 && a0 < b0 + 4ull * e.nb && b0 < a0 + 4ull * e.na);
+    if (direct && e.nn_clean) da = reinterpret_cast<uint32_t *>(e.nn_clean);
+    if (direct && e.nn_denoised) db = reinterpret_cast<uint32_t *>(e.nn_denoised);
     if (launch_evb_nearest(e.box_scratch, e.clean, e.na, e.denoised, e.nb, reinterpret_cast<float *>(da),
                            reinterpret_cast<float *>(db), &frame, e.ctr, e.spin_limit, num_sms, st))
       return -1;
@@ -454,7 +459,7 @@ int launch_eval_metrics(const EvalArgs &e, int num_sms, cudaStream_t st) {
   k_ev_sum<<<ra, kEvRedThreads, 0, st>>>(da, e.na, pa_sum);
   k_ev_sum<<<rb, kEvRedThreads, 0, st>>>(db, e.nb, pb_sum);
   k_ev_metrics<<<1, kEvFinThreads, 0, st>>>(pa_sum, ra, pb_sum, rb, red, ra, frame, e.na, e.nb, e.out);
-  if (!e.box_scratch) {
+  if (!direct) {
     if (e.nn_clean) cudaMemcpyAsync(e.nn_clean, da, 4ull * e.na, cudaMemcpyDeviceToDevice, st);
     if (e.nn_denoised) cudaMemcpyAsync(e.nn_denoised, db, 4ull * e.nb, cudaMemcpyDeviceToDevice, st);
   }
