@@ -429,9 +429,9 @@ int launch_eval_metrics(const EvalArgs &e, int num_sms, cudaStream_t st) {
   bool direct = false;
   if (e.box_scratch) {
     // the distances go where the caller wants them, unless one output lies over the other
-    // (the sums below read both)
+    // (the sums below read both) or is not aligned for stores of floats (a copy takes any address)
     const uintptr_t a0 = reinterpret_cast<uintptr_t>(e.nn_clean), b0 = reinterpret_cast<uintptr_t>(e.nn_denoised);
-    direct = !(a0 && b0 && a0 < b0 + 4ull * e.nb && b0 < a0 + 4ull * e.na);
+    direct = !(a0 && b0 && a0 < b0 + 4ull * e.nb && b0 < a0 + 4ull * e.na) && ((a0 | b0) & 3u) == 0;
     if (direct && e.nn_clean) da = reinterpret_cast<uint32_t *>(e.nn_clean);
     if (direct && e.nn_denoised) db = reinterpret_cast<uint32_t *>(e.nn_denoised);
     if (launch_evb_nearest(e.box_scratch, e.clean, e.na, e.denoised, e.nb, reinterpret_cast<float *>(da),
