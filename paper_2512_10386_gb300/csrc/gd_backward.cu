@@ -11,7 +11,7 @@
 //   dt/dgamma = -t * (d^2)^(gamma/2) * ln(d^2) / 2 / ((d^2)^(gamma/2) + eps_k)   (0 at d^2 = 0),
 //   dr/dF = -m(1-m)/(T F),  dr/dtau = m(1-m)/T,  m = sigmoid((ln F - tau)/T).
 // The forward leaves the three sums over a point's terms (TrainCache), so this pass
-// is one read of 41 bytes a point, bound by the FP64 pipe (two divisions a point).
+// is one read of 37 bytes a point, bound by the FP64 pipe (two divisions a point).
 // Measured, 560,000 points, K = 32: 1036 us with a pass over stored neighbour lists
 // -> 60 us.  Sums in FP64; the grid reduction is a fixed two-level tree, so the
 // result does not depend on scheduling.

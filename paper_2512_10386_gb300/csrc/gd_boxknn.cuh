@@ -466,7 +466,6 @@ __device__ __forceinline__ bool bk_knn(const Src &src, BkShared<KROW> &S, bool a
   const bool ties_only = cut.c_at > kSelBuf;
   const int32_t kbase = cut.lo + 1;
   const float lo_f = cut.lo >= 0 ? __int_as_float(cut.lo) : -1.0f, hi_f = __int_as_float(cut.hi);
-  const f32x2 LO2 = pk2(lo_f, lo_f), HI2 = pk2(hi_f, hi_f);
   uint32_t a = 0, np = 0;
   bk_traverse(src, qb, qx, qy, qz, hi_f, S.x, S.y, S.z, [&](uint32_t cur) {
     uint32_t gtlo = 0, gthi = 0;

@@ -675,20 +675,20 @@ __device__ __forceinline__ unsigned long long prefix_of(unsigned long long k, in
   return level == 0 ? 0ull : (k >> (63 - 3 * level));
 }
 
-// Binary searches over sorted keys; kb[idx - koff] is the key of sorted
-// position idx (kb = a shared-memory window starting at position koff, or the
-// global array with koff = 0).
+// Binary searches over sorted keys.
 // first index in [lo, hi) whose level-L prefix is >= pre
-__device__ __forceinline__ uint32_t lower_pre(const unsigned long long *kb, uint32_t koff, uint32_t lo,
-                                              uint32_t hi, unsigned long long pre, int level) {
+__device__ __forceinline__ uint32_t lower_pre(const unsigned long long *keys, uint32_t lo, uint32_t hi,
+                                              unsigned long long pre, int level) {
   while (lo < hi) {
     uint32_t mid = lo + ((hi - lo) >> 1);
-    if (prefix_of(kb[mid - koff], level) < pre) lo = mid + 1;
+    if (prefix_of(keys[mid], level) < pre) lo = mid + 1;
     else hi = mid;
   }
   return lo;
 }
-// first index in [lo, hi) whose level-L prefix is > pre
+// first index in [lo, hi) whose level-L prefix is > pre; kb[idx - koff] is the key of
+// sorted position idx (a shared-memory window starting at position koff, or the whole
+// array with koff = 0)
 __device__ __forceinline__ uint32_t upper_pre(const unsigned long long *kb, uint32_t koff, uint32_t lo,
                                               uint32_t hi, unsigned long long pre, int level) {
   while (lo < hi) {
@@ -715,22 +715,21 @@ constexpr uint32_t kLeavesSmemCap = (kLeavesSmemKeys - kLeavesPart) / 2 - 1;
 // Every search below stays within cap + 1 positions of i, except the one at the
 // maximum depth D (over `keys`, the whole frame's).  Returns the leaf's count and
 // level, or 0 if no leaf starts at i.
-__device__ __forceinline__ uint32_t find_leaf(const unsigned long long *kb, uint32_t koff,
-                                              const unsigned long long *keys, uint32_t i, uint32_t fb, uint32_t fe,
+__device__ __forceinline__ uint32_t find_leaf(const unsigned long long *keys, uint32_t i, uint32_t fb, uint32_t fe,
                                               uint32_t cap, int D, int DB, int *level) {
-  const unsigned long long ki = kb[i - koff];
+  const unsigned long long ki = keys[i];
   const uint32_t wlo = (i - fb > cap + 1) ? i - cap - 1 : fb, whi = (fe - i > cap + 1) ? i + cap + 1 : fe;
   // does the level-l node that holds i-1 and i have more than cap points?
   auto big = [&](int l) {
     if (l == 0) return (fe - fb) > cap;
     const unsigned long long pre = prefix_of(ki, l);
-    return upper_pre(kb, koff, i, whi, pre, l) - lower_pre(kb, koff, wlo, i, pre, l) > cap;
+    return upper_pre(keys, 0, i, whi, pre, l) - lower_pre(keys, wlo, i, pre, l) > cap;
   };
   int L;  // level of the first node that starts at i
   if (i == fb) {
     L = 0;
   } else {
-    const unsigned long long x = kb[i - 1 - koff] ^ ki;
+    const unsigned long long x = keys[i - 1] ^ ki;
     const int l = (x == 0) ? 21 : (__clzll((long long)x) - 1) / 3;  // shared levels below the root
     if (l >= D) return 0;                                            // same max-depth node
     // below level DB the keys are in octree order only inside level-DB nodes of more
@@ -744,7 +743,7 @@ __device__ __forceinline__ uint32_t find_leaf(const unsigned long long *kb, uint
     const unsigned long long pre = prefix_of(ki, L);
     uint32_t e;
     if (L < D) {
-      e = upper_pre(kb, koff, i, whi, pre, L);
+      e = upper_pre(keys, 0, i, whi, pre, L);
       if (e - i > cap) continue;
     } else {
       e = upper_pre(keys, 0, i, fe, pre, L);  // a max-depth node may be of any size
@@ -859,7 +858,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_leaves(const unsigned long lo
       s_cnt[it][threadIdx.x] = 0;
       if (i >= t.end) continue;
       int L = 0;
-      s_cnt[it][threadIdx.x] = find_leaf(keys, 0, keys, i, fb, fe, cap, D, DB, &L);
+      s_cnt[it][threadIdx.x] = find_leaf(keys, i, fb, fe, cap, D, DB, &L);
       s_lvl[it][threadIdx.x] = (uint8_t)L;
     }
   }
@@ -1172,7 +1171,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_front_small(const SmallArgs A
   for (uint32_t i0 = 0; i0 < n; i0 += kSmallThreads) {
     const uint32_t i = i0 + tid;
     int L = 0;
-    const uint32_t c = i < n ? find_leaf(buf, 0, buf, i, 0, n, A.cap, A.D, A.DB, &L) : 0u;
+    const uint32_t c = i < n ? find_leaf(buf, i, 0, n, A.cap, A.D, A.DB, &L) : 0u;
     const uint32_t m = __ballot_sync(0xFFFFFFFFu, c != 0);
     if (lane == 0) s_wsum[w] = m ? atomicAdd(&s_nl, (uint32_t)__popc(m)) : 0u;
     __syncwarp();

@@ -3,18 +3,20 @@
 //
 // Each CTA pulls octree leaves from a device work counter and runs, for one
 // leaf at a time, every per-leaf step of Sec. 3 in shared memory:
-//   extents and adaptive voxel size h (Eq. 10-11) -> voxel occupancy counts in a
-//   shared hash table with warp-aggregated atomics, voxel gate (Eq. 12) and
-//   compaction of P_1 -> kNN of every P_1 point against the leaf's P_1 (seeded
-//   register top-K, candidates broadcast from shared memory, ties broken by
-//   input index), r_K (Eq. 13) -> exact percentile gate
+//   (extents and adaptive voxel size h, Eq. 10-11, come from the prep kernel) ->
+//   voxel occupancy in counters addressed by the grid cell, or a hash table where
+//   the grid is large, with warp-aggregated atomics; voxel gate (Eq. 12) and
+//   compaction of P_1 -> kNN of every P_1 point against the leaf's P_1 (counting
+//   selection, gd_knn_select.cuh; candidates broadcast from shared memory, ties
+//   broken by input index), r_K (Eq. 13) -> exact percentile gate
 //   (Eq. 14) as a rank cut on r_K^2 -> median density (Eq. 16) -> dual-weight
 //   gravitational score (Eq. 15-21) -> Top-lambda or log-threshold selection,
 //   scattered to input order (Eq. 22).
 // The leaf's points arrive in shared memory by one TMA bulk copy
-// (cp.async.bulk + mbarrier).  Leaves larger than the shared-memory capacity
-// (only possible at max depth, i.e. with massive duplicates) run the same code
-// on a per-point spill area in global memory.
+// (cp.async.bulk + mbarrier).  Leaves larger than the shared-memory layout (leaf
+// capacities above 2,048 points, nodes at the maximum depth) run the same code
+// on a per-point spill area in global memory, or, where the call allows it, in
+// kernels over the whole GPU (gd_big.cu).
 //
 // FP32 steps that decide integers (voxel indices, neighbour order, the density
 // rank cut) use explicitly rounded intrinsics so no FMA contraction can change

@@ -1,7 +1,7 @@
 // gd_leaf_kernel.cuh -- device code of the fused per-leaf kernel, shared by the
-// two translation units that instantiate it (gd_leaf.cu: the plain path;
-// gd_leaf_rec.cu: the instantiation that also writes debug / training tensors).
-// Split so the two sets of instantiations compile in parallel.
+// translation units that instantiate it (gd_leaf.cu: the plain path; gd_leaf_rec.cu:
+// the instantiation that also writes debug / training tensors; gd_leaf_xl.cu: the
+// cross-leaf phases).  Split so the sets of instantiations compile in parallel.
 #pragma once
 
 #include <type_traits>
@@ -697,7 +697,7 @@ template <int kNT, typename IdxT, bool kRec, bool kXl>
 __device__ void process_leaf(const LeafArgs &A, const Leaf lf, const float4 *__restrict__ pts, const LeafMem &M,
                              LeafShared &S) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const uint32_t NT = blockDim.x, NW = NT >> 5;  // 64 or 128 threads (execution knob)
+  const uint32_t NT = blockDim.x, NW = NT >> 5;  // 64 to 512 threads (leaf_auto_threads, execution knob)
   const uint32_t nt = lf.count;
   const denoise_params &P = A.p;
   const uint32_t lt = lanemask_lt();

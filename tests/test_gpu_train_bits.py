@@ -8,7 +8,6 @@ scale where the products leave the range of FP32 the terms are summed in FP64: o
 rounding of 2^-53 for each term and three for its factors."""
 
 import math
-import os
 import struct
 import subprocess
 from fractions import Fraction
@@ -19,7 +18,6 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2512_10386_gb300", "csrc")
 POINTS, TERMS = 96, 31
 
 PROGRAM = r"""
