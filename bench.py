@@ -761,9 +761,9 @@ def run_serving(args):
 
 
 def run_batch_profile(args):
-    """The batched LiDAR workload alone (64 frames, K = 24, leaf capacity 128,
-    64-thread leaf CTAs: the autotuner's usual pick), W + K graph-captured
-    batches, for profiling the leaf kernel on it; prints one JSON line."""
+    """The batched LiDAR workload alone (64 frames, K = 24, leaf capacity 128 and the
+    default knobs: the autotuner's usual pick), W + K graph-captured batches, for
+    profiling the leaf kernels on it; prints one JSON line."""
     import dataclasses
 
     import torch
@@ -775,7 +775,6 @@ def run_batch_profile(args):
     offs = np.cumsum([0] + [len(f[0]) for f in frames]).tolist()
     xyz = torch.from_numpy(np.concatenate([f[0] for f in frames])).cuda()
     d = Denoiser(max_points=int(offs[-1]), max_frames=len(frames))
-    d.set_tuning(0, 0, 64)
     d.set_graphs(True)
     P = dataclasses.replace(Params(k=24), leaf_capacity=128)
     stream = torch.cuda.Stream()

@@ -13,8 +13,9 @@
 //
 // 500,000 against 510,000 points (two passes): 96.8 ms -> 0.95 ms, 0.77 ms of it the
 // four search kernels; counts within 8 % of the extent among 560,000 points: 73.0 ms
-// -> 2.27 ms.  The full pass is bound by the FP32 pipe; these by instruction issue of
-// the box tests and of the chunks that the spheres' borders cross.
+// -> 2.27 ms.  The full pass is bound by the FP32 pipe; these by the box tests and the
+// chunks that the spheres' borders cross: issue in 62 % (nearest) and 67 % (counts) of the
+// cycles with 37 and 41 % of the warp slots occupied, no one stall on top.
 #include "gd_boxes.cuh"
 #include "gd_f32x2.cuh"
 
