@@ -266,7 +266,7 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   // 248 us with 512 threads a leaf, 47 so)
   la.lmax = leaf_pick_lmax(p.leaf_capacity < c->frame_points ? p.leaf_capacity : c->frame_points, kmax,
                            c->smem_optin - 2048);
-  if (const uint32_t above = big_leaf_above(p, n, dbg != nullptr || c->training != 0)) {
+  if (const uint32_t above = big_leaf_above(p, n, c->frame_points, dbg != nullptr || c->training != 0)) {
     la.skip_big = 1;
     la.unit_start = c->d_vals[0];  // free after the front end, as the other key buffer
     la.far_queue = reinterpret_cast<uint2 *>(c->d_keys[front_sorted_buffer((int)p.max_depth, false) ^ 1]);

@@ -705,13 +705,15 @@ __global__ void __launch_bounds__(256) k_big_out(const LeafArgs A) {
 // capacity 1,000, 200k points 377 / 416, 560k 589 / 751; capacity 2,048, 10k 661 / 271,
 // 100k 937 / 376, 560k 1299 / 873.  Where a call is one leaf, its serial time on one
 // CTA decides: from 512 points.
-uint32_t big_leaf_above(const denoise_params &p, uint32_t n, bool rec) {
+// `frame`: points of the largest frame, which no leaf exceeds (64 frames of 600 points at
+// depth 1, judged by all their points: 11 launches for nothing, 172 us a call instead of 162).
+uint32_t big_leaf_above(const denoise_params &p, uint32_t n, uint32_t frame, bool rec) {
   if (p.stage_off || p.rescore_p2 || p.cross_leaf || rec) return 0;
   const uint32_t above = p.leaf_capacity >= n ? 512u : 1024u;
-  if (n <= above) return 0;
+  if (frame <= above) return 0;
   if (p.leaf_capacity > above) return above;
   // a depth limit that leaves more than `above` points to some cell
-  return (p.max_depth < 8 && (n >> (3 * p.max_depth)) > above) ? above : 0u;
+  return (p.max_depth < 8 && (frame >> (3 * p.max_depth)) > above) ? above : 0u;
 }
 
 int launch_big(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches) {

@@ -286,7 +286,7 @@ int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launc
 int launch_leaf(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches, cudaStream_t side = nullptr,
                 cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
 // The leaf size above which a call's leaves are taken by gd_big.cu's kernels (0: none).
-uint32_t big_leaf_above(const denoise_params &p, uint32_t n, bool rec);
+uint32_t big_leaf_above(const denoise_params &p, uint32_t n, uint32_t frame, bool rec);
 int launch_big(const LeafArgs &a, int num_sms, cudaStream_t st, int *launches);
 // the recording instantiation (debug / training outputs), in its own translation unit
 int launch_leaf_rec(const LeafArgs &a, int num_sms, cudaStream_t st);

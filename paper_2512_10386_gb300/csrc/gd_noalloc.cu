@@ -185,7 +185,7 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
   la.big_bpp = leaf_big_bpp(64);
   la.kmax = leaf_kmax(p->k);
   la.lmax = leaf_pick_lmax(p->leaf_capacity, la.kmax, su.smem_optin - 2048);
-  if (const uint32_t above = big_leaf_above(*p, nn, false)) {
+  if (const uint32_t above = big_leaf_above(*p, nn, nn, false)) {
     la.skip_big = 1;
     la.unit_start = fa.vals[0];  // free after the front end, as the other key buffer
     la.far_queue = reinterpret_cast<uint2 *>(fa.keys[front_sorted_buffer(fa.max_depth, false) ^ 1]);

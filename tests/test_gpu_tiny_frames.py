@@ -72,3 +72,22 @@ def test_leaf_finder_of_small_frames():
     search, whole = _stage(3000, 20, 8, 2), _stage(3000, 20, 2048, 2)
     print(search, whole)
     assert whole <= search, (search, whole)
+
+
+@pytest.mark.parametrize("kw", [{"max_depth": 1}, {"max_depth": 0}, {"leaf_capacity": 0xFFFFFFFF}, {"leaf_capacity": 2000}])
+def test_no_launches_for_leaves_that_cannot_be(kw):
+    """Whether a batch can hold large leaves is a question of its largest frame: 400 frames
+    of 500 points launch what 2 such frames launch."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2512_10386_gb300 import Denoiser, Params
+    n = {}
+    for frames in (2, 400):
+        x = _cloud(500 * frames, 3)
+        d = Denoiser(max_points=len(x), max_frames=frames)
+        try:
+            d.run_batch(x, [500 * i for i in range(frames + 1)], Params(k=8, **kw))
+            n[frames] = d.stats()["launches"]
+        finally:
+            d.close()
+    assert n[400] <= n[2] + 1, n  # (small leaves may take a launch of their own)
