@@ -241,6 +241,7 @@ int enqueue(denoise_ctx *c, const float *xyz_dev, uint32_t n, uint32_t nframes, 
   if (use_events) cudaEventRecord(c->ev[0], st);
   LeafArgs la{};
   la.n = n;
+  la.frame = c->frame_points;
   la.spts = c->d_spts;
   la.leaves = c->d_leaves;
   la.order = c->d_order;

@@ -212,6 +212,7 @@ int launch_front(const FrontArgs &a, cudaStream_t st, int *launches, cudaEvent_t
 
 struct LeafArgs {
   uint32_t n;                   // total points (bounds check of every output index)
+  uint32_t frame;               // points of the largest frame
   const float4 *spts;
   const Leaf *leaves;
   uint32_t *order;              // [n_leaves] leaf indices, largest class first (written by the prep step)

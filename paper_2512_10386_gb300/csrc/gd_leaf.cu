@@ -180,7 +180,17 @@ int launch_leaf_prep(const LeafArgs &a, int num_sms, cudaStream_t st, int *launc
 //                      200k 291 / 231 / 368, 300k 294 / 292 / 463, 560k 402 / 484 / 886
 //   1,024-point leaves: 200k 672 / 527 / 377, 300k 671 / 508 / 457, 560k 753 / 589 / 747
 //   2,048-point leaves: 10k 1184 / 838 / 661, 560k 2362 / 1612 / 1299
-static uint32_t leaf_auto_threads(uint32_t n, uint32_t lmax) {
+// A batch of many frames a little above the capacity has leaves of an eighth of a frame
+// (one octree level): where they are two or more an SM, the width is chosen for a sixth
+// of the largest frame.  us a call, by the capacity's size / so (capacity 512, 64 frames):
+// 600 points 175 / 128, 800 186 / 148, 1,300 207 / 168; 200 frames of 600 216 / 191.
+static uint32_t leaf_auto_threads(const LeafArgs &a, int num_sms) {
+  const uint32_t n = a.n;
+  uint32_t lmax = a.lmax;
+  if (lmax <= 512 && a.frame > a.p.leaf_capacity && 8ull * n >= 2ull * (uint32_t)num_sms * a.frame) {
+    const uint32_t size = pow2ceil(a.frame / 6u);
+    if (size < lmax) lmax = size;
+  }
   if (lmax <= 64) return 64;
   if (lmax <= 128) return 128;
   if (lmax <= 256) return n <= (64u << 10) ? 256 : 128;
@@ -208,7 +218,7 @@ int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launche
     // the big leaves' kernels on `st`; the other leaves, which need nothing of
     // theirs, beside them on the side stream where there is one
     const bool beside = side && fork && join;
-    if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a.n, a.lmax);
+    if (a.threads == 0 && a.ctas_per_sm == 0) a.threads = leaf_auto_threads(a, num_sms);
     if (launches) ++*launches;
     if (beside && (cudaEventRecord(fork, st) != cudaSuccess || cudaStreamWaitEvent(side, fork, 0) != cudaSuccess))
       return -1;
@@ -218,7 +228,7 @@ int launch_leaf(const LeafArgs &args, int num_sms, cudaStream_t st, int *launche
     return 0;
   }
   const bool chosen = a.threads == 0 && a.ctas_per_sm == 0;  // the caller leaves the choice open
-  if (chosen) a.threads = leaf_auto_threads(a.n, a.lmax);
+  if (chosen) a.threads = leaf_auto_threads(a, num_sms);
   if (a.xphase != 0) {  // the cross-leaf phases: their own instantiation
     if (launches) ++*launches;
     return launch_leaf_xl(a, num_sms, st);

@@ -172,6 +172,7 @@ extern "C" int denoise_run_noalloc(const float *xyz, size_t n, const denoise_par
   fa.leaf_capacity = p->leaf_capacity;
   LeafArgs la{};
   la.n = nn;
+  la.frame = nn;
   la.spts = fa.spts;
   la.leaves = fa.leaves;
   la.order = (uint32_t *)(b + kOffOrder);

@@ -91,3 +91,30 @@ def test_no_launches_for_leaves_that_cannot_be(kw):
         finally:
             d.close()
     assert n[400] <= n[2] + 1, n  # (small leaves may take a launch of their own)
+
+
+@pytest.mark.parametrize("m", [600, 800, 1300])
+def test_leaf_stage_of_frames_just_above_the_capacity(m):
+    """Frames of which one octree level makes leaves of less than half the capacity: the same
+    leaves under a capacity of 256 and 512, so about the same leaf stage (within a quarter)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    g = torch.Generator().manual_seed(9)
+    from paper_2512_10386_gb300 import Denoiser, Params
+    x = torch.rand(64 * m, 3, generator=g).cuda()
+    offs, ms = [i * m for i in range(65)], {}
+    d = Denoiser(max_points=len(x), max_frames=64)
+    try:
+        d.set_profiling(True)
+        masks = {}
+        for cap in (256, 512):
+            t = []
+            for _ in range(12):
+                masks[cap] = d.run_batch(x, offs, Params(k=12, leaf_capacity=cap)).mask
+                t.append(d.stats()["stage_ms"][4])
+            ms[cap] = sorted(t)[6]
+    finally:
+        d.close()
+    print(ms)
+    assert torch.equal(masks[256], masks[512])
+    assert ms[512] <= 1.25 * ms[256], ms
